@@ -3,6 +3,7 @@
 // k_ascent_trace.cu.  Internal to libubqp.  The design is described at the
 // top of k_ascent.cu.
 #pragma once
+#include <algorithm>
 #include <climits>
 
 #include "ubqp_internal.cuh"
@@ -26,12 +27,6 @@ __device__ __forceinline__ uint64_t globaltimer() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
-}
-
-// acc + d * (signed byte i of w), for d in {-1, +1}, in one dp4a: the second
-// operand holds d in byte i and zeros elsewhere.
-__device__ __forceinline__ int byte_sel(int i, int d) {
-  return (int)((unsigned)(d & 0xFF) << (8 * i));
 }
 
 // The R best entries (gain r.x, tag r.y) held one per lane across a warp,
@@ -59,17 +54,32 @@ __device__ __forceinline__ void runners_up(int2 r, int first, int* cand) {
   }
 }
 
-// Negate S and toggle the x bit of element ek (relinking: freeze it) with a
-// binary decision on ek: about log2(E) branches instead of E predicated ops.
+// Keys.  Element e of a thread keeps key = 32 gain + (31 - e % 32), so that an
+// integer maximum over up to 32 keys orders by gain, then by lower index
+// (|gain| < 2^23, so |key| < 2^28).  An element that is no candidate has
+// kOutKey; row updates move it by at most 2^13 per move, over at most 2^14
+// start-up rows and 2^14 relinking steps, so it never reaches a real key.
+constexpr int kKeyBits = 5;
+constexpr int kOutKey = -(1 << 30);
+
+// The flip of the owned element ek, found by a binary decision on its local
+// index (about log2(E) branches instead of E predicated operations): its key
+// becomes that of the gain -gain (relinking: it leaves the candidates) with
+// the element's own term of the row update that follows, -2 q_kk, taken off
+// beforehand, and its selector changes sign.
 template <int LO, int HI, int E, bool RL>
-__device__ __forceinline__ void flip_tree(int (&S)[E], int (&Ck)[E], int ek) {
+__device__ __forceinline__ void flip_tree(int (&key)[E], uint32_t (&sel)[E],
+                                          uint32_t (&xm)[(E + 31) / 32],
+                                          const int (&q)[E / 4], int ek, int gain) {
   if constexpr (HI - LO == 1) {
-    S[LO] = RL ? 0 : -S[LO];
-    Ck[LO] = RL ? INT_MIN : (Ck[LO] ^ 1);
+    const int qkk = (int)(int8_t)((unsigned)q[LO >> 2] >> (8 * (LO & 3)));
+    key[LO] = RL ? kOutKey : ((2 * qkk - gain) << kKeyBits) + (31 - (LO & 31));
+    sel[LO] ^= 0x80u << (8 * (LO & 3));
+    xm[LO >> 5] ^= 1u << (LO & 31);
   } else {
     constexpr int MID = (LO + HI) / 2;
-    if (ek < MID) flip_tree<LO, MID, E, RL>(S, Ck, ek);
-    else flip_tree<MID, HI, E, RL>(S, Ck, ek);
+    if (ek < MID) flip_tree<LO, MID, E, RL>(key, sel, xm, q, ek, gain);
+    else flip_tree<MID, HI, E, RL>(key, sel, xm, q, ek, gain);
   }
 }
 
@@ -203,6 +213,7 @@ struct RelinkArgs {
   int64_t* f_best;
   int32_t* dist;
   uint16_t* trace;
+  uint64_t* xs;  // W words of shared memory
 };
 
 // RL = false: steepest ascent of x_g in place (f_s updated, flips to flips_s).
@@ -217,72 +228,71 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
                                            int W, uint64_t* __restrict__ x_g,
                                            int64_t* __restrict__ f_s, int32_t max_flips,
                                            int32_t* __restrict__ flips_s,
-                                           unsigned* __restrict__ err, uint64_t* xs,
-                                           uint4* spec_slots,
+                                           unsigned* __restrict__ err, uint4* spec_slots,
                                            const float* __restrict__ y_g, G& grp,
                                            const RelinkArgs* rl = nullptr,
                                            uint16_t* __restrict__ trace_row = nullptr,
                                            int64_t trace_cap = 0) {
   constexpr int E = 16 * C;
-  constexpr int CW = 16 * T;  // indices per chunk
-  static_assert(E <= 32, "local index must fit 5 bits");
+  constexpr int NG = (E + 31) / 32;  // key groups
+  constexpr int CW = 16 * T;         // indices per chunk
   const int g = grp.rank();
+  // this thread's column offset in each chunk, 0 where the chunk lies beyond
+  // the row: those elements are no candidates, and what they read moves their
+  // keys by no more than a real row would.  Row offsets fit 32 bits (n and
+  // ldq <= 2^14).
+  const uint32_t ld32 = (uint32_t)ldq;
+  uint32_t off[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+    off[c] = c * CW + 16 * g < ldq ? (uint32_t)(c * CW + 16 * g) : 0u;
+  auto row_chunk = [&](int k, int c) {
+    return reinterpret_cast<const uint4*>(Q8 + ((uint32_t)k * ld32 + off[c]));
+  };
 
-  int y[E], S[E], Ck[E];
-  int ndiff = 0;  // relinking: owned variables where x and g differ
-  // ---- owned bits of x; C and S per element
+  int key[E];
+  uint32_t sel[E];  // +-64 in the element's byte: (1 - 2x) times the sign below
+  uint32_t xm[NG];  // x bits of the owned elements
+  uint32_t neg = 0;  // 0: sel is oriented for moves with d = +1, else for -1
+  int ndiff = 0;    // relinking: owned variables where x and g differ
+#pragma unroll
+  for (int h = 0; h < NG; ++h) xm[h] = 0;
+  // ---- owned bits of x, selectors, and keys from y = Q x of the tensor-core
+  // start-up (y_g, exact integers in fp32; without it the rows are added below)
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int j0 = c * CW + 16 * g;
-    uint32_t nib = 0, diff = 0xFFFFu;
+    uint32_t nib = 0, in = 0;
     if (j0 < n) {
-      nib = (uint32_t)((x_g[j0 >> 6] >> (j0 & 63)) & 0xFFFFull);
-      if (n - j0 < 16) nib &= (1u << (n - j0)) - 1u;
+      in = n - j0 < 16 ? (1u << (n - j0)) - 1u : 0xFFFFu;
+      nib = (uint32_t)(x_g[j0 >> 6] >> (j0 & 63)) & in;
       if (RL) {
-        uint32_t gn = (uint32_t)((rl->g[j0 >> 6] >> (j0 & 63)) & 0xFFFFull);
-        if (n - j0 < 16) gn &= (1u << (n - j0)) - 1u;
-        diff = nib ^ gn;
-        ndiff += __popc(diff);
+        in &= nib ^ (uint32_t)(rl->g[j0 >> 6] >> (j0 & 63));
+        ndiff += __popc(in);
       }
     }
+    xm[c >> 1] |= nib << (16 * (c & 1));
+    float4 y4[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      y4[v] = y_g && j0 < ldy ? reinterpret_cast<const float4*>(y_g + j0)[v]
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int o = 0; o < 16; ++o) {
       const int e = c * 16 + o, j = j0 + o;
-      const int xb = (int)((nib >> o) & 1u);
-      y[e] = 0;
-      if (j < n && ((diff >> o) & 1u)) {
-        const int qjj = Q8[(int64_t)j * ldq + j];
-        S[e] = xb ? -128 : 128;
-        Ck[e] = 64 * qjj + 2 * (31 - e) + xb;
-      } else {
-        S[e] = 0;
-        Ck[e] = INT_MIN;
-      }
-    }
-  }
-  // ---- y = Q x on the owned columns: from the tensor-core start-up when
-  // given (y_g, exact integers in fp32), else by adding the rows k with x_k = 1
-  if (y_g) {
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const int j0 = c * CW + 16 * g;
-      if (j0 < ldy) {
-        const float4* src = reinterpret_cast<const float4*>(y_g + j0);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const float4 t4 = src[v];
-          y[c * 16 + 4 * v + 0] = __float2int_rn(t4.x);
-          y[c * 16 + 4 * v + 1] = __float2int_rn(t4.y);
-          y[c * 16 + 4 * v + 2] = __float2int_rn(t4.z);
-          y[c * 16 + 4 * v + 3] = __float2int_rn(t4.w);
-        }
-      }
+      const bool xb = (nib >> o) & 1u, cd = (in >> o) & 1u;
+      const float4 yv = y4[o >> 2];
+      const float yf = (o & 3) == 0 ? yv.x : (o & 3) == 1 ? yv.y : (o & 3) == 2 ? yv.z : yv.w;
+      const int y2 = 2 * __float2int_rn(yf);
+      const int qjj = cd ? Q8[(int64_t)j * ldq + j] : 0;
+      key[e] = cd ? ((qjj + (xb ? -y2 : y2)) << kKeyBits) + (31 - (e & 31)) : kOutKey;
+      sel[e] = (xb ? 0xC0u : 0x40u) << (8 * (o & 3));
     }
   }
   for (int w = 0; w < W && !y_g; ++w) {
     uint64_t word = x_g[w] & valid_mask(n, w);
     while (word) {
-      constexpr int RF = C == 1 ? 4 : 2;  // rows in flight
+      constexpr int RF = C == 1 ? 4 : C == 2 ? 2 : 1;  // rows in flight
       int ks[RF];
       int nk = 0;
 #pragma unroll
@@ -299,10 +309,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       for (int r = 0; r < RF; ++r)
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          const int j0 = c * CW + 16 * g;
-          q[r][c] = (r < nk && j0 < ldq)
-                        ? __ldg(reinterpret_cast<const uint4*>(Q8 + (int64_t)ks[r] * ldq + j0))
-                        : make_uint4(0, 0, 0, 0);
+          q[r][c] = r < nk ? __ldg(row_chunk(ks[r], c)) : make_uint4(0, 0, 0, 0);
         }
 #pragma unroll
       for (int r = 0; r < RF; ++r)
@@ -311,14 +318,36 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
           const int wv[4] = {(int)q[r][c].x, (int)q[r][c].y, (int)q[r][c].z, (int)q[r][c].w};
 #pragma unroll
           for (int o = 0; o < 16; ++o)
-            y[c * 16 + o] = __dp4a(wv[o >> 2], byte_sel(o & 3, 1), y[c * 16 + o]);
+            key[c * 16 + o] = __dp4a(wv[o >> 2], (int)sel[c * 16 + o], key[c * 16 + o]);
         }
     }
   }
   // ---- first argmax
-  int kmax = INT_MIN;
+  int km[NG][2];
 #pragma unroll
-  for (int e = 0; e < E; ++e) kmax = max(kmax, Ck[e] + S[e] * y[e]);
+  for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = INT_MIN;
+#pragma unroll
+  for (int e = 0; e < E; e += 2)
+    km[e >> 5][(e >> 1) & 1] = __vimax3_s32(km[e >> 5][(e >> 1) & 1], key[e], key[e + 1]);
+  // the group's {max gain, 2k + x_k} from each thread's best key: the first
+  // key group that attains the thread's largest gain (lower groups hold lower
+  // indices)
+  auto reduce_key = [&]() {
+    int bk = max(km[0][0], km[0][1]), e0 = 31;
+    uint32_t xw = xm[0];
+#pragma unroll
+    for (int h = 1; h < NG; ++h) {
+      const int k = max(km[h][0], km[h][1]);
+      if (k > (bk | 31)) {
+        bk = k;
+        e0 = 32 * h + 31;
+        xw = xm[h];
+      }
+    }
+    const int l = 31 - (bk & 31), e = e0 - (bk & 31);
+    const int j = (e >> 4) * CW + 16 * g + (e & 15);
+    return grp.reduce(bk >> kKeyBits, (j << 1) | (int)((xw >> l) & 1u));
+  };
   // Speculation: the next move is often the runner-up of the previous
   // reduction (about 40% of moves at n = 7000), so each move copies this
   // thread's chunks of the runner-up rows (prow) into its own shared-memory
@@ -333,18 +362,14 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   // slot (buffer b, row i, chunk c) of thread g at plane ((b RR + i) C + c):
   // planes of T x 16 bytes, threads side by side, so a warp's copies and
   // reads cover all banks without conflicts
-  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(spec_slots) + (uint32_t)g * 16;
+  const uint32_t slot0 =
+      R > 0 ? (uint32_t)__cvta_generic_to_shared(spec_slots) + (uint32_t)g * 16 : 0u;
   int buf = 0;
-  auto reduce_key = [&](int kt) {
-    const int gain = kt >> 6;
-    const int e = 31 - ((kt >> 1) & 31);
-    const int j = (e >> 4) * CW + 16 * g + (e & 15);
-    return grp.reduce(gain, (j << 1) | (kt & 1));
-  };
-  int2 best = reduce_key(kmax);
+  int2 best = reduce_key();
 
   int64_t fval = *f_s;
   int flips = 0;
+  if (max_flips == 0) max_flips = INT_MAX;
   // relinking: path length, best intermediate value and its step
   const int dist = RL ? grp.sum(ndiff) : 0;
   int64_t fbest = fval;
@@ -354,8 +379,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     if (RL) {
       if (flips >= dist - 1) break;  // the last step only reaches g
     } else {
-      if (max_flips > 0 && flips >= max_flips) break;
-      if (best.x <= 0) break;
+      if (best.x <= 0 || flips >= max_flips) break;
     }
     if ((flips & 1023) == 1023) {
       const bool late = (int64_t)(globaltimer() - t0) > kTimeoutNs;
@@ -365,8 +389,6 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       }
     }
     const int k = best.y >> 1;
-    const int d = (best.y & 1) ? -1 : 1;  // 1 - 2 x_k before the flip
-    const int dsel[4] = {byte_sel(0, d), byte_sel(1, d), byte_sel(2, d), byte_sel(3, d)};
     fval += best.x;
     ++flips;
     if (RL) {
@@ -379,12 +401,12 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     if constexpr (TR) {  // the move record: flipped indices in order
       if (g == 0 && flips <= trace_cap) trace_row[flips - 1] = (uint16_t)k;
     }
-    uint4 q[C];
+    int q[4 * C];
     bool hit = false;
     if constexpr (R > 0) {
       int hi = -1;
 #pragma unroll
-      for (int i = 0; i < R; ++i)
+      for (int i = 0; i < RR; ++i)
         if (prow[i] == k) hi = i;
       if (hi >= 0) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -392,18 +414,20 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
 #pragma unroll
         for (int c = 0; c < C; ++c)
           asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(q[c].x), "=r"(q[c].y), "=r"(q[c].z), "=r"(q[c].w)
+                       : "=r"(q[4 * c]), "=r"(q[4 * c + 1]), "=r"(q[4 * c + 2]),
+                         "=r"(q[4 * c + 3])
                        : "r"(a + (uint32_t)(c * T * 16)));
         hit = true;
       }
     }
     if (!hit) {
-      const int8_t* row = Q8 + (int64_t)k * ldq;
 #pragma unroll
       for (int c = 0; c < C; ++c) {
-        const int j0 = c * CW + 16 * g;
-        q[c] = j0 < ldq ? __ldg(reinterpret_cast<const uint4*>(row + j0))
-                        : make_uint4(0, 0, 0, 0);
+        const uint4 v = __ldg(row_chunk(k, c));
+        q[4 * c] = (int)v.x;
+        q[4 * c + 1] = (int)v.y;
+        q[4 * c + 2] = (int)v.z;
+        q[4 * c + 3] = (int)v.w;
       }
     }
     if constexpr (R > 0) {  // fetch the runners-up's rows for the next move
@@ -416,11 +440,8 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
         prow[i] = r < n ? r : -1;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          const int j0 = c * CW + 16 * g;
-          // chunks at or beyond ldq are not copied: their elements have
-          // S = 0, so whatever the slot holds never changes a key
-          if (prow[i] >= 0 && j0 < ldq) {
-            const int8_t* src = Q8 + (int64_t)prow[i] * ldq + j0;
+          if (prow[i] >= 0) {
+            const uint4* src = row_chunk(prow[i], c);
             const uint32_t a = slot0 + (uint32_t)((buf * RR + i) * C + c) * (T * 16);
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src)
                          : "memory");
@@ -430,28 +451,30 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       asm volatile("cp.async.commit_group;" ::: "memory");
       buf ^= 1;
     }
-    // the owner of k flips x_k: negate S_k, toggle the x bit in C_k (when
-    // relinking, k leaves the candidates instead: S_k = 0, C_k = INT_MIN)
+    // orient the selectors for this move's d = 1 - 2 x_k (they are kept as
+    // the last move left them: the signs of successive moves agree about
+    // every other time)
+    const uint32_t ng = (uint32_t)(best.y & 1);
+    if (ng != neg) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) sel[e] ^= 0x80u << (8 * (e & 3));
+      neg = ng;
+    }
+    // the owner of k flips x_k (when relinking, k leaves the candidates)
     const int kc = k / CW, kr = k - kc * CW;
     if ((kr >> 4) == g) {
       const int ek = kc * 16 + (kr & 15);
-      flip_tree<0, E, E, RL>(S, Ck, ek);
+      flip_tree<0, E, E, RL>(key, sel, xm, q, ek, best.x);
     }
-    int km[4] = {INT_MIN, INT_MIN, INT_MIN, INT_MIN};
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const int wv[4] = {(int)q[c].x, (int)q[c].y, (int)q[c].z, (int)q[c].w};
+    for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = INT_MIN;
 #pragma unroll
-      for (int o = 0; o < 16; o += 2) {
-        const int e = c * 16 + o;
-        y[e] = __dp4a(wv[o >> 2], dsel[o & 3], y[e]);
-        y[e + 1] = __dp4a(wv[o >> 2], dsel[(o + 1) & 3], y[e + 1]);
-        km[(o >> 1) & 3] = __vimax3_s32(km[(o >> 1) & 3], Ck[e] + S[e] * y[e],
-                                        Ck[e + 1] + S[e + 1] * y[e + 1]);
-      }
+    for (int e = 0; e < E; e += 2) {
+      key[e] = __dp4a(q[e >> 2], (int)sel[e], key[e]);
+      key[e + 1] = __dp4a(q[e >> 2], (int)sel[e + 1], key[e + 1]);
+      km[e >> 5][(e >> 1) & 1] = __vimax3_s32(km[e >> 5][(e >> 1) & 1], key[e], key[e + 1]);
     }
-    kmax = max(max(km[0], km[1]), max(km[2], km[3]));
-    best = reduce_key(kmax);
+    best = reduce_key();
   }
   // copies still in flight must land before the slots serve another start
   if (R > 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -461,6 +484,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       *rl->f_best = fbest;
       if (rl->dist) *rl->dist = dist;
     }
+    uint64_t* xs = rl->xs;
     for (int w = g; w < W; w += T) xs[w] = x_g[w];
     grp.sync();
     for (int t = g; t < tbest; t += T) {
@@ -477,19 +501,14 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     *f_s = fval;
     if (flips_s) *flips_s = flips;
   }
-  for (int w = g; w < W; w += T) xs[w] = 0;
-  grp.sync();
+  grp.sync();  // every thread has read its words of x_g
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int j0 = c * CW + 16 * g;
-    uint64_t bits = 0;
-#pragma unroll
-    for (int o = 0; o < 16; ++o) bits |= (uint64_t)(Ck[c * 16 + o] & 1 & (S[c * 16 + o] != 0)) << o;
-    if (bits) atomicOr(reinterpret_cast<unsigned long long*>(&xs[j0 >> 6]),
-                       (unsigned long long)(bits << (j0 & 63)));
+    if (j0 < 64 * W)
+      reinterpret_cast<uint16_t*>(x_g)[j0 >> 4] =
+          (uint16_t)(xm[c >> 1] >> (16 * (c & 1)));
   }
-  grp.sync();
-  for (int w = g; w < W; w += T) x_g[w] = xs[w];
   grp.sync();
 }
 
@@ -514,7 +533,6 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                     unsigned long long* __restrict__ next, uint16_t* __restrict__ trace,
                     int64_t ldt, int64_t cnt_lo, int64_t cnt_hi) {
   __shared__ int2 rec[2][T / 32];
-  __shared__ uint64_t xs[UBQP_MAX_N / 64];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
@@ -538,7 +556,7 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
       continue;
     }
     ascend_one<T, C, R, false, TR>(Q8, ldq, ldy, n, W, X + (int64_t)s * W, f + s, max_flips,
-                                   flips ? flips + s : nullptr, err, xs, spec_slots,
+                                   flips ? flips + s : nullptr, err, spec_slots,
                                    Y ? Y + t * ldy : nullptr, grp, nullptr,
                                    TR ? trace + (int64_t)s * ldt : nullptr, ldt);
   }
@@ -552,7 +570,6 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
                     const int64_t* __restrict__ n_items, int32_t max_flips,
                     unsigned long long* __restrict__ next) {
   __shared__ int2 rec[2][T / 32];
-  __shared__ uint64_t xs[UBQP_MAX_N / 64];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
@@ -578,7 +595,7 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
       continue;
     }
     ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s, max_flips,
-                     b.flips ? b.flips + s : nullptr, b.err, xs, spec_slots,
+                     b.flips ? b.flips + s : nullptr, b.err, spec_slots,
                      b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
   }
 }
@@ -595,7 +612,7 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
 // boundaries.
 template <int T, int C, int R, int TS>
 __device__ __forceinline__ void climb_item(const BatchDesc* __restrict__ d, int2 it,
-                                           int32_t max_flips, int2* rec_flat, uint64_t* xs,
+                                           int32_t max_flips, int2* rec_flat,
                                            uint4* spec_slots, int sg) {
   const BatchDesc& b = d[it.x];
   if (b.err[1] != 0) return;  // Q failed its symmetry check: no climb
@@ -607,12 +624,12 @@ __device__ __forceinline__ void climb_item(const BatchDesc* __restrict__ d, int2
   if constexpr (TS == T) {
     Group<T> grp{reinterpret_cast<int2 (*)[T / 32]>(rec_flat), 0};
     ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s, max_flips,
-                        b.flips ? b.flips + s : nullptr, b.err, xs, spec_slots,
+                        b.flips ? b.flips + s : nullptr, b.err, spec_slots,
                         b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
   } else if constexpr (TS == 32) {  // one warp per start: warp-level reductions only
     Group<32> grp;
     ascend_one<32, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
-                         max_flips, b.flips ? b.flips + s : nullptr, b.err, xs + sg * (32 * C / 4),
+                         max_flips, b.flips ? b.flips + s : nullptr, b.err,
                          spec_slots + sg * spec_slot_count<32, C, R>(),
                          b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
   } else {
@@ -620,7 +637,7 @@ __device__ __forceinline__ void climb_item(const BatchDesc* __restrict__ d, int2
                      sg * TS, 1 + sg};
     ascend_one<TS, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
                          max_flips, b.flips ? b.flips + s : nullptr, b.err,
-                         xs + sg * (TS * C / 4), spec_slots + sg * spec_slot_count<TS, C, R>(),
+                         spec_slots + sg * spec_slot_count<TS, C, R>(),
                          b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
   }
 }
@@ -633,7 +650,7 @@ template <int T, int C, int R, int TS>
 __device__ __forceinline__ void climb_class(const BatchDesc* __restrict__ d,
                                             const int2* __restrict__ items, int4 range,
                                             int32_t max_flips, unsigned long long* next,
-                                            int2* rec_flat, uint64_t* xs, uint4* spec_slots,
+                                            int2* rec_flat, uint4* spec_slots,
                                             long long* slot) {
   constexpr int K = T / TS;
   const int sg = (int)threadIdx.x / TS, r = (int)threadIdx.x % TS;
@@ -652,7 +669,7 @@ __device__ __forceinline__ void climb_class(const BatchDesc* __restrict__ d,
       sg_sync();  // every thread has read slot[sg] before its leader writes it again
     }
     if (t >= range.y) break;
-    climb_item<T, C, R, TS>(d, items[range.x + t], max_flips, rec_flat, xs, spec_slots, sg);
+    climb_item<T, C, R, TS>(d, items[range.x + t], max_flips, rec_flat, spec_slots, sg);
   }
 }
 
@@ -663,46 +680,47 @@ ascent_batch_packed_kernel(const BatchDesc* __restrict__ d, const int2* __restri
                            unsigned long long* __restrict__ next) {
   static_assert(T / 8 == 32, "sub-groups down to one warp");
   __shared__ int2 rec_flat[2 * (T / 32)];
-  __shared__ uint64_t xs[T * C / 4];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
   __shared__ long long slot[8];
-  climb_class<T, C, R, T>(d, items, ranges[0], max_flips, next ? next : nullptr, rec_flat, xs,
+  climb_class<T, C, R, T>(d, items, ranges[0], max_flips, next ? next : nullptr, rec_flat,
                           spec_slots, slot);
   __syncthreads();
   climb_class<T, C, R, T / 2>(d, items, ranges[1], max_flips, next ? next + 1 : nullptr,
-                              rec_flat, xs, spec_slots, slot);
+                              rec_flat, spec_slots, slot);
   __syncthreads();
   climb_class<T, C, R, T / 4>(d, items, ranges[2], max_flips, next ? next + 2 : nullptr,
-                              rec_flat, xs, spec_slots, slot);
+                              rec_flat, spec_slots, slot);
   __syncthreads();
   climb_class<T, C, R, T / 8>(d, items, ranges[3], max_flips, next ? next + 3 : nullptr,
-                              rec_flat, xs, spec_slots, slot);
+                              rec_flat, spec_slots, slot);
 }
 
-// Four independent warps per block, one start each (n <= 512); a
-// programmatic dependent like the block kernel.
-template <int C, int R, bool TR>
-__global__ void __launch_bounds__(128)
+// Independent warps, one start each (kWarps per block); counts, starts and
+// launch as in the block kernel, the first wave one warp per block over the
+// whole grid before any block's second warp.
+constexpr int kWarps = 2;
+template <int C, int R, bool TR, int OCC>
+__global__ void __launch_bounds__(32 * kWarps, OCC)
 ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                    uint64_t* __restrict__ X, int64_t* __restrict__ f,
                    const int32_t* __restrict__ idx, const int64_t* __restrict__ count,
                    int64_t S, int32_t max_flips, int32_t* __restrict__ flips,
                    const float* __restrict__ Y, int64_t ldy, unsigned* __restrict__ err,
                    unsigned long long* __restrict__ next, uint16_t* __restrict__ trace,
-                   int64_t ldt) {
-  __shared__ uint64_t xs_all[4][16];
-  __shared__ uint4 spec_slots[4 * spec_slot_count<32, C, R>()];
+                   int64_t ldt, int64_t cnt_lo, int64_t cnt_hi) {
+  __shared__ uint4 spec_slots[kWarps * spec_slot_count<32, C, R>()];
   Group<32> grp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait();  // no early release: see pdl_release
   if (err[1] != 0) return;  // Q failed its symmetry check: no climb
   const int64_t cnt = *count;
+  if (cnt < cnt_lo || cnt > cnt_hi) return;  // another launch's counts
   auto take = [&](int64_t t) -> int64_t {  // the warp's next start (see the block kernel)
-    if (t < 0) return (int64_t)blockIdx.x * 4 + warp;
-    if (!next) return t + (int64_t)gridDim.x * 4;
+    if (t < 0) return (int64_t)warp * gridDim.x + blockIdx.x;
+    if (!next) return t + (int64_t)gridDim.x * kWarps;
     unsigned long long v = 0;
     if (lane == 0) v = atomicAdd(next, 1ull);
-    return (int64_t)gridDim.x * 4 + (int64_t)__shfl_sync(0xffffffffu, v, 0);
+    return (int64_t)gridDim.x * kWarps + (int64_t)__shfl_sync(0xffffffffu, v, 0);
   };
   for (int64_t t = take(-1); t < cnt; t = take(t)) {
     const int s = idx[t];
@@ -711,7 +729,7 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
       continue;
     }
     ascend_one<32, C, R, false, TR>(Q8, ldq, ldy, n, W, X + (int64_t)s * W, f + s, max_flips,
-                                    flips ? flips + s : nullptr, err, xs_all[warp],
+                                    flips ? flips + s : nullptr, err,
                                     spec_slots + warp * spec_slot_count<32, C, R>(),
                                     Y ? Y + t * ldy : nullptr, grp, nullptr,
                                     TR ? trace + (int64_t)s * ldt : nullptr, ldt);
@@ -722,8 +740,8 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
 // intermediate solution to Xb[p], its value to fb[p], the distance to dist[p]
 // (may be NULL).  trace: P rows of ldt uint16 scratch.  Y: y = Q X[p] rows from
 // the tensor-core start-up, or NULL.
-template <int T, int C, int R>
-__global__ void __launch_bounds__(T, 1)
+template <int T, int C, int R, int OCC>
+__global__ void __launch_bounds__(T, OCC)
 relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                     const uint64_t* __restrict__ X, const int64_t* __restrict__ f,
                     const uint64_t* __restrict__ G, int64_t P, uint64_t* __restrict__ Xb,
@@ -750,10 +768,10 @@ relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
   };
   for (int64_t p = take(-1); p < P; p = take(p)) {
     const RelinkArgs a{G + p * W, Xb + p * W, fb + p, dist ? dist + p : nullptr,
-                       trace + p * ldt};
+                       trace + p * ldt, xs};
     int64_t f0 = f[p];
     ascend_one<T, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
-                              nullptr, err, xs, spec_slots, Y ? Y + p * ldy : nullptr, grp, &a);
+                              nullptr, err, spec_slots, Y ? Y + p * ldy : nullptr, grp, &a);
   }
 }
 
@@ -780,10 +798,10 @@ relink_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
   };
   for (int64_t p = take(-1); p < P; p = take(p)) {
     const RelinkArgs a{G + p * W, Xb + p * W, fb + p, dist ? dist + p : nullptr,
-                       trace + p * ldt};
+                       trace + p * ldt, xs_all[warp]};
     int64_t f0 = f[p];
     ascend_one<32, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
-                               nullptr, err, xs_all[warp],
+                               nullptr, err,
                                spec_slots + warp * spec_slot_count<32, C, R>(),
                                Y ? Y + p * ldy : nullptr, grp, &a);
   }
@@ -801,84 +819,76 @@ int resident_grid(K kernel, int threads, int sm_count) {
   return per_sm * sm_count;
 }
 
-template <int T, int C, bool TR, int OCC>
-cudaError_t launch_block_occ(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
-                             const int64_t* count, int64_t S, int32_t max_flips, int32_t* flips,
-                             const float* Y, unsigned long long* next, uint16_t* trace,
-                             int64_t ldt, int64_t cnt_lo, int64_t cnt_hi, cudaStream_t st) {
-  int grid = resident_grid(ascent_block_kernel<T, C, kSpecRows, TR, OCC>, T, h->sm_count);
-  if ((int64_t)grid > S) grid = (int)S;
-  return launch_pdl(ascent_block_kernel<T, C, kSpecRows, TR, OCC>, dim3(grid), dim3(T), 0, st,
-                    h->Q8, h->ldq, h->n, h->W, X, f, idx, count, S, max_flips, flips, Y,
-                    (int64_t)h->n_tc, h->err, next, trace, ldt, cnt_lo, cnt_hi);
-}
+// One ascent launch of a group shape: T threads and 16 C elements per thread
+// for each start (T = 32: one warp, kWarps to a block), R runner-up rows
+// copied ahead, registers sized for OCC blocks per SM.  Climbs only for counts
+// in [lo, hi].
+struct AscArgs {
+  const ubqp_q* h;
+  uint64_t* X;
+  int64_t* f;
+  const int32_t* idx;
+  const int64_t* count;
+  int64_t S;
+  int32_t max_flips;
+  int32_t* flips;
+  const float* Y;
+  unsigned long long* next;
+  uint16_t* trace;
+  int64_t ldt;
+  cudaStream_t st;
+};
+template <int T, int C, int R, int OCC, bool TR>
+struct Climb {
+  static constexpr int kBlock = T == 32 ? 32 * kWarps : T;
+  static constexpr int kPer = kBlock / T;  // starts per block
+  // starts resident on the device at once
+  static int64_t capacity(const ubqp_q* h) { return (int64_t)kPer * blocks(h); }
+  static int64_t blocks(const ubqp_q* h) {
+    if constexpr (T == 32)
+      return resident_grid(ascent_warp_kernel<C, R, TR, OCC>, kBlock, h->sm_count);
+    else
+      return resident_grid(ascent_block_kernel<T, C, R, TR, OCC>, kBlock, h->sm_count);
+  }
+  static cudaError_t launch(const AscArgs& a, int64_t lo, int64_t hi) {
+    const dim3 grid((unsigned)std::min<int64_t>(blocks(a.h), (a.S + kPer - 1) / kPer));
+    if constexpr (T == 32)
+      return launch_pdl(ascent_warp_kernel<C, R, TR, OCC>, grid, dim3(kBlock), 0, a.st, a.h->Q8,
+                        a.h->ldq, a.h->n, a.h->W, a.X, a.f, a.idx, a.count, a.S, a.max_flips,
+                        a.flips, a.Y, (int64_t)a.h->n_tc, a.h->err, a.next, a.trace, a.ldt, lo,
+                        hi);
+    else
+      return launch_pdl(ascent_block_kernel<T, C, R, TR, OCC>, grid, dim3(kBlock), 0, a.st,
+                        a.h->Q8, a.h->ldq, a.h->n, a.h->W, a.X, a.f, a.idx, a.count, a.S,
+                        a.max_flips, a.flips, a.Y, (int64_t)a.h->n_tc, a.h->err, a.next, a.trace,
+                        a.ldt, lo, hi);
+  }
+};
 
-// Block groups, registers sized for one block per SM: with at most one listed
-// start per SM every start climbs alone on its SM, and this gives the shortest
-// chain (measured at n = 7000: 1.91 ms for the ~52 passers of 1000 random
-// starts, against 2.14 ms with registers sized for two).  The smaller groups
-// (64 and 128 threads) still fit several blocks per SM.  Climbs only for
-// counts up to cnt_hi; returns its resident capacity (blocks per SM x SMs).
-template <int T, int C, bool TR>
-cudaError_t launch_block(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
-                         const int64_t* count, int64_t S, int32_t max_flips, int32_t* flips,
-                         const float* Y, unsigned long long* next, uint16_t* trace, int64_t ldt,
-                         int64_t cnt_hi, cudaStream_t st) {
-  return launch_block_occ<T, C, TR, 1>(h, X, f, idx, count, S, max_flips, flips, Y, next, trace,
-                                       ldt, 0, cnt_hi, st);
-}
-template <int T, int C, bool TR>
-int64_t block_capacity(const ubqp_q* h) {
-  return resident_grid(ascent_block_kernel<T, C, kSpecRows, TR, 1>, T, h->sm_count);
-}
-
-// With more listed starts than the one-block-per-SM launch holds at once,
-// several blocks per SM overlap one chain's waits with the others' work:
-// groups of two 16-index chunks per thread, the fewest threads that hold n,
-// and as many blocks per SM as their registers allow (measured, 1000 starts
-// all climbed: n = 2000 0.94 vs 1.25 ms, 3000 2.02 vs 2.97, 4000 3.17 vs 4.02,
-// 6000 7.29 vs 8.63; n = 5000 with 8192 diversified starts, ~4500 passing:
-// 9.6 vs 13.5 ms).  Up to n = 1024 the one-block-per-SM groups, six per SM,
-// are faster at every count, and so are 256-thread groups above n = 6144.
-// The count is known only on the device, so for a list that may exceed the
-// capacity both launches are made; each climbs only for its own range of
-// counts and the other returns at once.
-template <bool TR>
-cudaError_t launch_block_many(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
-                              const int64_t* count, int64_t S, int32_t max_flips,
-                              int32_t* flips, const float* Y, unsigned long long* next,
-                              uint16_t* trace, int64_t ldt, int64_t cnt_lo, cudaStream_t st) {
-  const int n = h->n;
-#define UBQP_MANY(TT, OCC)                                                                   \
-  return launch_block_occ<TT, 2, TR, OCC>(h, X, f, idx, count, S, max_flips, flips, Y, next, \
-                                          trace, ldt, cnt_lo, INT64_MAX, st)
-  if (n <= 2048) UBQP_MANY(64, 8);
-  if (n <= 3072) UBQP_MANY(96, 5);
-  if (n <= 4096) UBQP_MANY(128, 4);
-  if (n <= 5120) UBQP_MANY(160, 3);
-  if (n <= 6144) UBQP_MANY(192, 2);
-  if (n <= 8192) UBQP_MANY(256, 2);
-#undef UBQP_MANY
-  return cudaErrorInvalidValue;
-}
-
-template <int C, bool TR>
-cudaError_t launch_warp(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
-                        const int64_t* count, int64_t S, int32_t max_flips, int32_t* flips,
-                        const float* Y, unsigned long long* next, uint16_t* trace, int64_t ldt,
-                        cudaStream_t st) {
-  int grid = resident_grid(ascent_warp_kernel<C, kSpecRows, TR>, 128, h->sm_count);
-  const int64_t need = (S + 3) / 4;
-  if ((int64_t)grid > need) grid = (int)need;
-  return launch_pdl(ascent_warp_kernel<C, kSpecRows, TR>, dim3(grid), dim3(128), 0, st, h->Q8,
-                    h->ldq, h->n, h->W, X, f, idx, count, S, max_flips, flips, Y,
-                    (int64_t)h->n_tc, h->err, next, trace, ldt);
-}
-
-// One ascent launch over the listed starts, with the group shape that holds
-// n; for 1024 < n <= 8192 and a list that may be longer than that launch's
-// resident capacity, also the several-blocks-per-SM launch, the two splitting
-// the counts at the capacity.
+// The ascent launches over the listed starts, by n and by how many of them
+// there are.  The count is known only on the device, so for a list that may
+// exceed a shape's range several launches are made, each climbing only for its
+// own range of counts; the others return at once (about 2 us).
+//   few  the shortest chain of moves: enough threads to hold n with 16 (32
+//        above n = 2560) elements each, runner-up rows copied, registers for as
+//        many blocks per SM as that leaves; for lists up to its resident
+//        capacity.
+//   mid  two chunks per thread and several blocks per SM, whose waits cover
+//        one another.
+//   all  the fewest warps that hold n (one up to n = 2048) without runner-up
+//        copies, for lists that keep every SM busy: there the issue slots
+//        bound the climb, and the copies cost more than their hits save.
+// Measured on 1000 to 12 000 diversified starts, the passing ones climbed (us,
+// before -> now): n = 1025, 510 starts 187 -> 143; 2500, 542 starts 533 -> 359;
+// 1000, 5638 starts 784 -> 411; 1400, 6069: 1382 -> 701; 2000, 4214: 1406 ->
+// 967; 2500, 3213: 2082 -> 1343; 4000, 2193: 3046 -> 2091; 5000, 4469: 9080 ->
+// 5433; 6000, 2187: 7464 -> 3727; 7000, 54: 1857 -> 1697; 7000, 641: 3364 ->
+// 2663; 7000, 2172: 9610 -> 6535.  The boundary between mid and all lies where
+// a list of that n keeps mid's SMs busy anyway: both take the same time near
+// 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000 starts 2178
+// and 2077), earlier where mid fits only two or three blocks (n = 4800, 600
+// starts: 2387 mid, 2397 all; n = 5800, 300: 2620 and 2682, 600: 3612 and
+// 3000).
 template <bool TR>
 cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
                                  const int64_t* count, int64_t S, int32_t max_flips,
@@ -890,22 +900,42 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
     cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
   }
-#define UBQP_ASC_ARGS h, X, f, idx, count, S, max_flips, flips, Y, next, trace, ldt
-  if (n <= 256) return launch_warp<1, TR>(UBQP_ASC_ARGS, st);
-  if (n <= 512) return launch_warp<2, TR>(UBQP_ASC_ARGS, st);
-  if (n <= 1024) return launch_block<64, 1, TR>(UBQP_ASC_ARGS, INT64_MAX, st);
-  if (n > 8192) return launch_block<512, 2, TR>(UBQP_ASC_ARGS, INT64_MAX, st);
-  const int64_t cap = n <= 2048 ? block_capacity<128, 1, TR>(h)
-                      : n <= 4096 ? block_capacity<256, 1, TR>(h)
-                                  : block_capacity<256, 2, TR>(h);
-  const bool many = S > cap;
-  const int64_t hi = many ? cap : INT64_MAX;
-  cudaError_t e = n <= 2048   ? launch_block<128, 1, TR>(UBQP_ASC_ARGS, hi, st)
-                  : n <= 4096 ? launch_block<256, 1, TR>(UBQP_ASC_ARGS, hi, st)
-                              : launch_block<256, 2, TR>(UBQP_ASC_ARGS, hi, st);
-  if (e != cudaSuccess || !many) return e;
-  return launch_block_many<TR>(UBQP_ASC_ARGS, cap + 1, st);
-#undef UBQP_ASC_ARGS
+  const AscArgs a{h, X, f, idx, count, S, max_flips, flips, Y, next, trace, ldt, st};
+  // few: the shortest chain of moves, for lists up to its resident capacity;
+  // mid: several blocks per SM, whose waits cover one another; all: no
+  // runner-up copies and the fewest warps per start, for lists that keep the
+  // whole chip busy (more than `full` starts)
+  auto tiers = [&](auto few, auto mid, auto all, int64_t full) {
+    const int64_t cap = std::min(few.capacity(h), full);
+    cudaError_t e = few.launch(a, 0, cap);
+    if (e == cudaSuccess && cap < full && S > cap) e = mid.launch(a, cap + 1, full);
+    if (e == cudaSuccess && S > full) e = all.launch(a, full + 1, INT64_MAX);
+    return e;
+  };
+  auto two = [&](auto few, auto all, int64_t full) {
+    cudaError_t e = few.launch(a, 0, full);
+    if (e == cudaSuccess && S > full) e = all.launch(a, full + 1, INT64_MAX);
+    return e;
+  };
+  const int64_t full = 10ll * h->sm_count;
+#define UBQP_C(TT, CC, RR, OCC) Climb<TT, CC, RR, OCC, TR>{}
+  if (n <= 512) return two(UBQP_C(32, 1, 1, 8), UBQP_C(32, 1, 0, 10), full);
+  if (n <= 1024) return two(UBQP_C(64, 1, 1, 8), UBQP_C(32, 2, 0, 8), full);
+  if (n <= 1536) return tiers(UBQP_C(96, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 3, 0, 7), full);
+  if (n <= 2048) return tiers(UBQP_C(128, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 4, 0, 5), full);
+  if (n <= 2560) return tiers(UBQP_C(160, 1, 1, 3), UBQP_C(96, 2, 1, 4), UBQP_C(64, 3, 0, 7), full);
+  if (n <= 3072) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(96, 2, 1, 4), UBQP_C(64, 3, 0, 7), full);
+  if (n <= 4096) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(128, 2, 1, 4), UBQP_C(64, 4, 0, 5), full);
+  if (n <= 5120)
+    return tiers(UBQP_C(160, 2, 1, 1), UBQP_C(160, 2, 1, 3), UBQP_C(96, 4, 0, 3), 4ll * h->sm_count);
+  if (n <= 6144)
+    return tiers(UBQP_C(192, 2, 1, 1), UBQP_C(192, 2, 1, 2), UBQP_C(96, 4, 0, 3), 2ll * h->sm_count);
+  if (n <= 7168)
+    return tiers(UBQP_C(224, 2, 1, 1), UBQP_C(256, 2, 1, 2), UBQP_C(128, 4, 0, 3), full);
+  if (n <= 8192)
+    return tiers(UBQP_C(256, 2, 1, 1), UBQP_C(256, 2, 1, 2), UBQP_C(128, 4, 0, 3), full);
+  return UBQP_C(512, 2, 1, 1).launch(a, 0, INT64_MAX);
+#undef UBQP_C
 }
 
 template <int T, int C>
@@ -920,14 +950,14 @@ cudaError_t launch_ascent_batch_tc(const BatchDesc* d, const int2* items, const 
   return cudaGetLastError();
 }
 
-template <int T, int C>
+template <int T, int C, int OCC>
 cudaError_t launch_relink_block(const ubqp_q* h, const uint64_t* X, const int64_t* f,
                                 const uint64_t* G, int64_t P, uint64_t* Xb, int64_t* fb,
                                 int32_t* dist, uint16_t* trace, int64_t ldt, const float* Y,
                                 unsigned long long* next, cudaStream_t st) {
-  int grid = resident_grid(relink_block_kernel<T, C, kSpecRows>, T, h->sm_count);
+  int grid = resident_grid(relink_block_kernel<T, C, kSpecRows, OCC>, T, h->sm_count);
   if ((int64_t)grid > P) grid = (int)P;
-  relink_block_kernel<T, C, kSpecRows><<<grid, T, 0, st>>>(
+  relink_block_kernel<T, C, kSpecRows, OCC><<<grid, T, 0, st>>>(
       h->Q8, h->ldq, h->n, h->W, X, f, G, P, Xb, fb, dist, trace, ldt, Y, h->n_tc, h->err,
       next);
   return cudaGetLastError();

@@ -6,27 +6,37 @@
 // and a flip of bit k (d = 1 - 2 x_k before the flip) changes y by d times
 // column k of Q (= row k, Q being symmetric) and negates the sign of x_k.
 //
-// Design.  A group of T threads owns one start at a time (one warp for
-// n <= 512, else one block).  Thread g owns E = 16*C elements, in chunks of 16
+// Design.  A group of T threads owns one start at a time (one warp, or one
+// block of several).  Thread g owns E = 16*C elements, in chunks of 16
 // consecutive indices: element e lives at j = (e/16)*16T + 16g + e%16, so one
 // move loads row k of the int8 Q (= column k, Q being symmetric) with C fully
 // coalesced 16-byte loads per thread.  Per element the thread keeps, in
 // registers,
-//     y_j,   S_j = 128 (1 - 2 x_j),   C_j = 64 Q_jj + 2 (31 - e) + x_j,
-// so that the argmax key  key_j = C_j + S_j y_j = 64 Delta_j + 2 (31 - e) + x_j
-// costs one multiply-add.  A move is therefore, per element: y += d q as one
-// dp4a (d placed in the coefficient's byte lane), key = C + S y, and a running
-// max kept in four independent chains.  The key orders by gain, then by lower
-// index inside the thread, and carries x_j in its low bit; across threads the
-// group reduces (gain, 2j + x) with warp max/min reductions (redux.sync), so
-// every thread learns k, x_k and Delta_k.  The thread owning k negates S_k and
-// toggles the x bit of C_k.  Rows are read from L2 (the int8 Q of one
-// instance, e.g. 49 MB at n = 7000, stays resident there); nothing per move
-// goes to HBM.  The chain of moves is latency-bound: per move a dependent L2
-// row fetch, the update and a block-wide reduction.  The fetch is taken off
-// the chain when the move was predicted: every move also copies the row of
-// the reduction's runner-up into shared memory, and the next move is that
-// row often enough (about 40% at n = 7000) to pay for the copies.
+//     key_j = 32 Delta_j + (31 - e%32)   and   sel_j = +-64 in j's byte lane,
+// the sign of sel_j being (1 - 2 x_j) d for the move at hand.  A move is then,
+// per element, one dp4a (key += 64 (1 - 2 x_j) d q_kj) and half a three-way
+// max: no y is kept, and no multiply-add forms the key.  When d changes sign
+// from one move to the next the selectors are flipped (one XOR each, about
+// every other move).  Measured against y, S and C registers with a dp4a, a
+// multiply-add and half a max per element (3 registers, 2.5 instructions):
+// 2 registers, so more starts fit an SM, and about 2 instructions, the ALU
+// pipe (XOR, max) and the FMA pipe (dp4a) sharing them.  The key orders by
+// gain, then by lower index inside the thread (up to 32 elements; larger
+// threads keep one maximum per 32); across threads the group reduces (gain,
+// 2j + x) with warp max/min reductions (redux.sync), so every thread learns k,
+// x_k and Delta_k.  The thread owning k resets key_k to -Delta_k, turns sel_k
+// and flips its x bit.  Rows are read from L2 (the int8 Q of one instance,
+// e.g. 49 MB at n = 7000, stays resident there); nothing per move goes to HBM.
+//
+// What bounds it.  With few starts the chain of moves is latency-bound: per
+// move a dependent L2 row fetch, the update and a block-wide reduction (n =
+// 7000, 54 starts: 791 cycles per move, 1.70 ms; 863 and 1.85 before).  The
+// fetch is taken off the chain when the move was predicted: every move also
+// copies the row of the reduction's runner-up into shared memory, and the next
+// move is that row often enough (about 40% at n = 7000) to pay for the copies.
+// With many starts the issue slots bound it (n = 1400, 6069 starts: 190 warp
+// instructions per move, 101 cycles per move and SM, 0.70 ms; 199 cycles and
+// 1.38 ms before).  launch_ascent_shaped picks the group shape by n and count.
 //
 // Start-up: y = Q x of every listed start comes from the tensor-core product of
 // the ascent workspace when given (exact integers in fp32), else each group
@@ -44,15 +54,31 @@ cudaError_t launch_relink(const ubqp_q* h, const uint64_t* X, const int64_t* f, 
     cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
   }
-#define UBQP_RL_ARGS h, X, f, G, P, Xb, fb, dist, trace, ldt, Y, next, st
-  if (n <= 256) return launch_relink_warp<1>(UBQP_RL_ARGS);
-  if (n <= 512) return launch_relink_warp<2>(UBQP_RL_ARGS);
-  if (n <= 1024) return launch_relink_block<64, 1>(UBQP_RL_ARGS);
-  if (n <= 2048) return launch_relink_block<128, 1>(UBQP_RL_ARGS);
-  if (n <= 4096) return launch_relink_block<256, 1>(UBQP_RL_ARGS);
-  if (n <= 8192) return launch_relink_block<256, 2>(UBQP_RL_ARGS);
-  if (n <= 16384) return launch_relink_block<512, 2>(UBQP_RL_ARGS);
-#undef UBQP_RL_ARGS
+  // P is known here: up to one pair per SM the registers are sized for one
+  // block per SM (the shortest chain), above it for two (n = 5000, 256 pairs:
+  // see the launch rule of the ascent)
+  const bool wide = P > h->sm_count;
+#define UBQP_RL(TT, CC, OCC) \
+  return launch_relink_block<TT, CC, OCC>(h, X, f, G, P, Xb, fb, dist, trace, ldt, Y, next, st)
+  if (n <= 512) return launch_relink_warp<1>(h, X, f, G, P, Xb, fb, dist, trace, ldt, Y, next, st);
+  if (n <= 1024) UBQP_RL(64, 1, 4);
+  if (n <= 2048) UBQP_RL(128, 1, 3);
+  if (n <= 2560) UBQP_RL(160, 1, 3);
+  if (n <= 4096) UBQP_RL(128, 2, 2);
+  if (n <= 5120) {
+    if (wide) UBQP_RL(160, 2, 2);
+    UBQP_RL(160, 2, 1);
+  }
+  if (n <= 7168) {
+    if (wide) UBQP_RL(224, 2, 2);
+    UBQP_RL(224, 2, 1);
+  }
+  if (n <= 8192) {
+    if (wide) UBQP_RL(256, 2, 2);
+    UBQP_RL(256, 2, 1);
+  }
+  if (n <= 16384) UBQP_RL(512, 2, 1);
+#undef UBQP_RL
   return cudaErrorInvalidValue;
 }
 
