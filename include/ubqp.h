@@ -390,8 +390,8 @@ int ubqp_solve_rounds(const ubqp_q* q, const ubqp_params* p, int32_t R, uint64_t
  * the tensor-core evaluation are one launch each for all instances (the
  * evaluation one persistent launch over the work units of every instance) or,
  * as the tuner decides, per-instance launches on internal streams; the
- * screen, the ascent of every passing start of every instance (one persistent
- * launch, largest instances first) and the best-of are one launch each; the
+ * screen and the best-of are one launch each, the ascent of every passing
+ * start of every instance one persistent launch or one per size class; the
  * start-up products y = Q x of the passing starts run per instance on the
  * internal streams.  Each instance's result is bit-identical to ubqp_solve on
  * that instance alone.
@@ -404,12 +404,9 @@ int ubqp_solve_rounds(const ubqp_q* q, const ubqp_params* p, int32_t R, uint64_t
  *   when there is one.
  * ubqp_batch_tune -- the autotuner: times the run for the candidate ascent
  *   group shapes (threads x chunks that hold the largest n, one start per
- *   group, or packed: 256-thread blocks climbing up to eight starts at once
- *   in sub-groups of 32, 64, 128 or 256 threads, the smallest that holds the
- *   instance's n, each taking its next start as soon as its climb ends; the
- *   instances too large for half a block climb in launches of their own
- *   beside it), the
- *   evaluation paths, one merged launch for the start generation and the
+ *   group, or packed: a launch per size class of the instances, each with the
+ *   group shape for its n, on the internal streams, the instances above
+ *   n = 4096 in launches of their own beside them), the evaluation paths, one merged launch for the start generation and the
  *   tensor-core evaluation of all instances (one persistent launch over the
  *   work units of every instance, largest first) or one launch per instance,
  *   the evaluation's schedule (at most 16, 12 or 8 K steps of 64 per work
@@ -460,10 +457,10 @@ int ubqp_batch_get(const ubqp_batch* b, int32_t i, uint64_t* best_x_dev, int64_t
  * in arrival order, every waiting request that fits -- up to max_batch
  * requests whose device memory fits the budget -- and runs them as one batch:
  * per-request upload, preparation, start generation and evaluation on the
- * lane's streams, then one shared launch each for the screen, the climb of
- * every passing start of every request (one persistent launch, several small
- * starts per block; requests too large for half a block climb in launches of
- * their own beside it) and the best-of.  Requests that arrive while batches run
+ * lane's streams, then a shared launch for the screen, the climb of every
+ * passing start of every request (one launch per size class; requests above
+ * n = 4096 in launches of their own beside them) and a shared launch for the
+ * best-of.  Requests that arrive while batches run
  * are taken together by the next free lane, so batches grow with the load,
  * and the lanes' batches overlap on the GPU.  Request memory comes from the
  * device's stream-ordered pool.  The paper solves one instance per run;

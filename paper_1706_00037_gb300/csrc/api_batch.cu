@@ -16,9 +16,10 @@
 // first, and for the start-up one unpacking launch and one persistent product
 // over the merged full-square work list, units past an instance's passing
 // count skipped on the device.
-// The climb is either one start per group of the plan's shape, or packed: a
-// 256-thread block climbs up to four starts of one instance at once in
-// sub-groups of 64 or 128 threads when the instance's n fits them.
+// The climb is either one start per group of the plan's shape, or packed: one
+// launch per size class of the instances, each with the group shape for its n,
+// and a launch of its own for every instance above the last class, all on the
+// internal streams.
 // The whole run can be captured into a CUDA graph and replayed (the seed lives
 // in device memory so a replay can use a new one).  An autotuner times, on the
 // batch itself, the candidate ascent group shapes (plain and packed), the
@@ -69,7 +70,7 @@ struct ubqp_batch {
   std::vector<size_t> scratch_bytes;
   std::vector<TmaDesc> mapA;             // TMA descriptor of each scratch
   int4* d_units = nullptr;               // packed ascent: the item range of each class
-  int64_t* d_nunits = nullptr;           // the item count, then the four class counters
+  int64_t* d_nunits = nullptr;           // the item count, then the class counters
   unsigned long long* d_next = nullptr;  // per instance: the start counter of its own climb
   // evaluation schedules: per instance, chunk tables of at most 8 and 12 K steps
   // (the handle's own table has 16)
@@ -187,32 +188,38 @@ int run_body(ubqp_batch* b, cudaStream_t st) {
   }
   // ---- one launch each: work list, every climb, every best
   if (b->packed) {
-    // instances too large for half a block climb in launches of their own on
-    // the fork streams, beside the packed launch of the others
-    const bool own = ubqp::packed_own_climb(b->max_n, b->asc_T, b->asc_C);
-    UBQP_BCUDA(ubqp::launch_batch_units(b->d_desc, b->d_order, b->count, b->asc_T, b->asc_C,
-                                        own, b->d_items, b->d_units, b->d_nunits, st));
-    if (own) {
-      UBQP_BCUDA(cudaEventRecord(b->ev_fork, st));
-      for (int k = 0; k < K; ++k) UBQP_BCUDA(cudaStreamWaitEvent(b->streams[k], b->ev_fork, 0));
-      for (int k = 0, j = 0; k < b->count; ++k) {
-        const int i = b->order[k];
-        const ubqp_q* q = b->qs[i];
-        if (!ubqp::packed_own_climb(q->n, b->asc_T, b->asc_C)) continue;
-        const ubqp::BatchDesc& d = b->h_desc[i];
-        UBQP_BCUDA(ubqp::launch_ascent(q, d.X, d.f, d.idx, d.count, p.num_starts, p.max_flips,
-                                       d.flips, d.Y, b->d_next + i, b->streams[j++ % K]));
+    // on the fork streams: the instances above the last class in launches of
+    // their own, then one launch per class that the batch has, largest first
+    // (the item count is followed by the class counters)
+    unsigned long long* next = reinterpret_cast<unsigned long long*>(b->d_nunits + 1);
+    UBQP_BCUDA(cudaMemsetAsync(next, 0, ubqp::kPackedClasses * sizeof(unsigned long long), st));
+    UBQP_BCUDA(ubqp::launch_batch_units(b->d_desc, b->d_order, b->count, b->d_items, b->d_units,
+                                        b->d_nunits, st));
+    UBQP_BCUDA(cudaEventRecord(b->ev_fork, st));
+    for (int k = 0; k < K; ++k) UBQP_BCUDA(cudaStreamWaitEvent(b->streams[k], b->ev_fork, 0));
+    int j = 0;
+    int64_t most[ubqp::kPackedClasses] = {}, all = 0;
+    for (int k = 0; k < b->count; ++k) {
+      const int i = b->order[k];
+      const ubqp_q* q = b->qs[i];
+      const ubqp::BatchDesc& d = b->h_desc[i];
+      if (!ubqp::packed_own_climb(q->n)) {
+        most[ubqp::packed_class(q->n)] += p.num_starts;
+        all += p.num_starts;
+        continue;
       }
+      UBQP_BCUDA(ubqp::launch_ascent(q, d.X, d.f, d.idx, d.count, p.num_starts, p.max_flips,
+                                     d.flips, d.Y, b->d_next + i, b->streams[j++ % K]));
     }
-    // the class counters: the words after the item count
-    UBQP_BCUDA(ubqp::launch_ascent_batch_packed(
-        b->d_desc, b->d_items, b->d_units, b->asc_T, b->asc_C, p.max_flips, b->asc_grid,
-        reinterpret_cast<unsigned long long*>(b->d_nunits + 1), st));
-    if (own)
-      for (int k = 0; k < K; ++k) {
-        UBQP_BCUDA(cudaEventRecord(b->ev_join[k], b->streams[k]));
-        UBQP_BCUDA(cudaStreamWaitEvent(st, b->ev_join[k], 0));
-      }
+    for (int c = ubqp::kPackedClasses - 1; c >= 0; --c)
+      if (most[c] > 0)
+        UBQP_BCUDA(ubqp::launch_ascent_batch_packed(b->d_desc, b->d_items, b->d_units, c,
+                                                    b->d_nunits, most[c], all, p.max_flips,
+                                                    b->sm_count, next, b->streams[j++ % K]));
+    for (int k = 0; k < K; ++k) {
+      UBQP_BCUDA(cudaEventRecord(b->ev_join[k], b->streams[k]));
+      UBQP_BCUDA(cudaStreamWaitEvent(st, b->ev_join[k], 0));
+    }
   } else {
     UBQP_BCUDA(ubqp::launch_batch_items(b->d_desc, b->d_order, b->count, b->d_items,
                                         b->d_nitems, st));
@@ -241,8 +248,7 @@ int set_shape(ubqp_batch* b, int T, int C, bool packed = false) {
   b->asc_T = T;
   b->asc_C = C;
   b->packed = packed;
-  b->asc_grid = packed ? ubqp::ascent_packed_grid(T, C, b->sm_count)
-                       : ubqp::ascent_batch_grid(T, C, b->sm_count);
+  b->asc_grid = packed ? 0 : ubqp::ascent_batch_grid(T, C, b->sm_count);
   return UBQP_OK;
 }
 
@@ -305,8 +311,9 @@ int ubqp_batch_create(const ubqp_q* const* qs, int32_t count, const ubqp_params*
   const size_t o_order = take(sizeof(int32_t) * count);
   const size_t o_items = take(sizeof(int2) * (size_t)S * count);
   const size_t o_nitems = take(16);
-  const size_t o_units = take(std::max<size_t>(sizeof(int4) * (size_t)S * count, 4 * sizeof(int4)));
-  const size_t o_nunits = take(5 * sizeof(int64_t));  // item count, one start counter per class
+  const size_t o_units = take(ubqp::kPackedClasses * sizeof(int4));
+  // item count, one start counter per class
+  const size_t o_nunits = take((1 + ubqp::kPackedClasses) * sizeof(int64_t));
   const size_t o_next = take(sizeof(unsigned long long) * (size_t)count);
   const size_t o_seed = take(16);
   // the merged evaluation: instances, tensor maps, work lists
@@ -589,13 +596,15 @@ int ubqp_batch_tune(ubqp_batch* b, void* stream) {
       if (t < cur) { cur = t; bt = sh[0]; bc = sh[1]; bp = false; }
     }
     if ((r = set_shape(b, bt, bc))) goto done;
-    // the packed ascent (sub-groups of 256, 128 or 64 threads by n)
+    // the packed ascent: a launch per size class (256 x 1 and 256 x 2 name the
+    // same climb; the first that holds the largest n)
     for (int c : {1, 2}) {
-      if (16 * 256 * c < b->max_n || 16 * 256 * c > 4 * std::max(b->max_n, 1024)) continue;
+      if (16 * 256 * c < b->max_n) continue;
       if ((r = set_shape(b, 256, c, true))) goto done;
       float t = 0;
       if ((r = time_run(&t))) goto done;
       if (t < cur) { cur = t; bt = 256; bc = c; bp = true; }
+      break;
     }
     if ((r = set_shape(b, bt, bc, bp))) goto done;
   }

@@ -12,9 +12,9 @@
 //     preparation, start generation and evaluation;
 //   one launch screens every request of the batch;
 //   per request: the tensor-core start-up y = Q x of its passing starts;
-//   one persistent launch climbs every passing start of every request of the
-//     batch (the packed climb of the batch plans: several small starts per
-//     block), one launch takes every request's best;
+//   one launch per size class of the requests climbs their passing starts (the
+//     packed climb of the batch plans; the largest requests in launches of
+//     their own), one launch takes every request's best;
 //   the results come back and the batch's requests complete together.
 // Requests that arrive while batches run wait for the next free lane, which
 // takes all of them at once, so the batches grow with the load; the lanes'
@@ -83,7 +83,7 @@ struct ServerLane {
   int32_t* d_order = nullptr;
   int2* d_items = nullptr;
   int4* d_units = nullptr;
-  int64_t* d_nitems = nullptr;  // the item count, then the start counter(s): one per class packed
+  int64_t* d_nitems = nullptr;  // the item count, then one start counter per class
   std::thread th;
 };
 
@@ -92,9 +92,6 @@ struct ubqp_server {
   int device = 0;
   int max_batch = kDefaultMaxBatch;
   int sm_count = 0;
-  int asc_T = 256, asc_C = 1;
-  bool packed = true;
-  int asc_grid = 0;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
   std::deque<Request*> queue;
@@ -270,36 +267,36 @@ int run_batch(ubqp_server* s, ServerLane& L, std::vector<Slot*>& live) {
                                       sl.mapA.bytes));
   }
   if ((st = join())) return st;
-  // ---- one persistent launch climbs every passing start of the batch
+  // ---- the packed climb of every passing start of the batch, on the fork
+  // streams: the requests above the last class in launches of their own, then
+  // one launch per class, largest first
   unsigned long long* next = reinterpret_cast<unsigned long long*>(L.d_nitems + 1);
-  if (s->packed) {
-    // requests too large for half a block climb in launches of their own on
-    // the fork streams, beside the packed launch of the others
-    const bool own = ubqp::packed_own_climb(live[L.h_order[0]]->r->n, s->asc_T, s->asc_C);
-    LCUDA(ubqp::launch_batch_units(L.d_desc, L.d_order, m, s->asc_T, s->asc_C, own, L.d_items,
-                                   L.d_units, L.d_nitems, L.st));
-    if (own) {
-      if ((st = fork())) return st;
-      for (int k = 0, j = 0; k < m; ++k) {
-        const int i = L.h_order[k];
-        Slot& sl = *live[i];
-        if (!ubqp::packed_own_climb(sl.h->n, s->asc_T, s->asc_C)) continue;
-        const ubqp::BatchDesc& d = L.h_desc[i];
-        const ReqLayout RL = req_layout(c, sl.h->n);
-        // the climb's start counter: past the small results
-        auto* cnt = reinterpret_cast<unsigned long long*>(sl.buf + RL.small + kClimbCounter);
-        LCUDA(ubqp::launch_ascent(sl.h, d.X, d.f, d.idx, d.count, S, p.max_flips, d.flips, d.Y,
-                                  cnt, L.fork[j++ % kForkStreams]));
-      }
+  LCUDA(cudaMemsetAsync(next, 0, ubqp::kPackedClasses * sizeof(unsigned long long), L.st));
+  LCUDA(ubqp::launch_batch_units(L.d_desc, L.d_order, m, L.d_items, L.d_units, L.d_nitems, L.st));
+  if ((st = fork())) return st;
+  int64_t most[ubqp::kPackedClasses] = {}, all = 0;
+  int j = 0;
+  for (int k = 0; k < m; ++k) {
+    const int i = L.h_order[k];
+    Slot& sl = *live[i];
+    if (!ubqp::packed_own_climb(sl.h->n)) {
+      most[ubqp::packed_class(sl.h->n)] += S;
+      all += S;
+      continue;
     }
-    LCUDA(ubqp::launch_ascent_batch_packed(L.d_desc, L.d_items, L.d_units, s->asc_T, s->asc_C,
-                                           p.max_flips, s->asc_grid, next, L.st));
-    if (own && (st = join())) return st;
-  } else {
-    LCUDA(ubqp::launch_batch_items(L.d_desc, L.d_order, m, L.d_items, L.d_nitems, L.st));
-    LCUDA(ubqp::launch_ascent_batch(L.d_desc, L.d_items, L.d_nitems, s->asc_T, s->asc_C,
-                                    p.max_flips, s->asc_grid, next, L.st));
+    const ubqp::BatchDesc& d = L.h_desc[i];
+    const ReqLayout RL = req_layout(c, sl.h->n);
+    // the climb's start counter: past the small results
+    auto* cnt = reinterpret_cast<unsigned long long*>(sl.buf + RL.small + kClimbCounter);
+    LCUDA(ubqp::launch_ascent(sl.h, d.X, d.f, d.idx, d.count, S, p.max_flips, d.flips, d.Y, cnt,
+                              L.fork[j++ % kForkStreams]));
   }
+  for (int cl = ubqp::kPackedClasses - 1; cl >= 0; --cl)
+    if (most[cl] > 0)
+      LCUDA(ubqp::launch_ascent_batch_packed(L.d_desc, L.d_items, L.d_units, cl, L.d_nitems,
+                                             most[cl], all, p.max_flips, s->sm_count, next,
+                                             L.fork[j++ % kForkStreams]));
+  if ((st = join())) return st;
   LCUDA(ubqp::launch_best_batch(L.d_desc, m, L.st));
   // ---- results back
   const int32_t Wmax = (c.max_n + 63) / 64;
@@ -446,8 +443,7 @@ int make_lane(ubqp_server* s, ServerLane* L) {
   const size_t o_order = rup(sizeof(ubqp::BatchDesc) * B, 256);
   const size_t o_items = o_order + rup(sizeof(int32_t) * B, 256);
   const size_t o_units = o_items + rup(sizeof(int2) * (size_t)S * B, 256);
-  const size_t o_cnt =
-      o_units + rup(std::max<int64_t>(sizeof(int4) * (size_t)S * B, 4 * sizeof(int4)), 256);
+  const size_t o_cnt = o_units + rup(ubqp::kPackedClasses * sizeof(int4), 256);
   if (cudaMalloc(&L->dmem, o_cnt + 256) != cudaSuccess) return UBQP_ERR_NOMEM;
   L->d_desc = (ubqp::BatchDesc*)(L->dmem + o_desc);
   L->d_order = (int32_t*)(L->dmem + o_order);
@@ -486,21 +482,6 @@ int ubqp_server_create(const ubqp_server_config* cfg, ubqp_server** out) {
     return sfail(UBQP_ERR_CUDA, "device query failed");
   if (s->cfg.memory_budget == 0)
     s->cfg.memory_budget = (int64_t)request_bytes(s->cfg, s->cfg.max_n) * s->cfg.workers;
-  // the batch climb: packed 256-thread blocks up to n = 8192, one start per
-  // 512-thread block beyond
-  if (cfg->max_n <= 4096) {
-    s->asc_T = 256;
-    s->asc_C = 1;
-  } else if (cfg->max_n <= 8192) {
-    s->asc_T = 256;
-    s->asc_C = 2;
-  } else {
-    s->asc_T = 512;
-    s->asc_C = 2;
-    s->packed = false;
-  }
-  s->asc_grid = s->packed ? ubqp::ascent_packed_grid(s->asc_T, s->asc_C, s->sm_count)
-                          : ubqp::ascent_batch_grid(s->asc_T, s->asc_C, s->sm_count);
   // keep freed pool memory cached so admissions never return to the OS allocator
   cudaMemPool_t pool;
   if (cudaDeviceGetDefaultMemPool(&pool, s->device) == cudaSuccess) {

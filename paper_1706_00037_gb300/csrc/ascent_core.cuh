@@ -148,63 +148,6 @@ struct Group {
   }
 };
 
-// TS consecutive threads of a larger block owning one start (TS >= 64, a
-// multiple of 32): the block-group operations of Group<TS> on the named
-// barrier `bar` (1..15) instead of the block-wide one, so that several
-// sub-groups of one block climb different starts independently.
-__device__ __forceinline__ void named_sync(int bar, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ bool named_or(int bar, int count, bool p) {
-  uint32_t out;
-  asm volatile(
-      "{\n .reg .pred pi, po;\n setp.ne.u32 pi, %1, 0;\n"
-      " bar.red.or.pred po, %2, %3, pi;\n selp.u32 %0, 1, 0, po;\n}\n"
-      : "=r"(out)
-      : "r"((uint32_t)p), "r"(bar), "r"(count)
-      : "memory");
-  return out != 0;
-}
-
-template <int TS>
-struct SubGroup {
-  static constexpr int NW = TS / 32;
-  int2 (*rec)[NW];  // [2][NW] shared, this sub-group's
-  int parity;
-  int base;  // first thread of the sub-group
-  int bar;   // its named barrier
-  __device__ __forceinline__ int rank() const { return (int)threadIdx.x - base; }
-  int2 mine;
-  __device__ __forceinline__ int2 reduce(int gain, int jx) {
-    const int lane = threadIdx.x & 31, warp = rank() >> 5;
-    const int m = __reduce_max_sync(0xffffffffu, gain);
-    const int c = __reduce_min_sync(0xffffffffu, gain == m ? jx : INT_MAX);
-    if (lane == 0) rec[parity][warp] = make_int2(m, c);
-    named_sync(bar, TS);
-    const int2 r = lane < NW ? rec[parity][lane] : make_int2(INT_MIN, INT_MAX);
-    const int m2 = __reduce_max_sync(0xffffffffu, r.x);
-    const int c2 = __reduce_min_sync(0xffffffffu, r.x == m2 ? r.y : INT_MAX);
-    parity ^= 1;
-    mine = r;
-    return make_int2(m2, c2);
-  }
-  template <int R>
-  __device__ __forceinline__ void runners(int first, int* cand) const {
-    runners_up<R>(mine, first, cand);
-  }
-  __device__ __forceinline__ bool any(bool p) { return named_or(bar, TS, p); }
-  __device__ __forceinline__ void sync() { named_sync(bar, TS); }
-  __device__ __forceinline__ int sum(int v) {
-    const int lane = threadIdx.x & 31, warp = rank() >> 5;
-    const int sv = __reduce_add_sync(0xffffffffu, v);
-    if (lane == 0) rec[parity][warp] = make_int2(sv, 0);
-    named_sync(bar, TS);
-    const int r = lane < NW ? rec[parity][lane].x : 0;
-    parity ^= 1;
-    return __reduce_add_sync(0xffffffffu, r);
-  }
-};
-
 // Path relinking of one pair (see relink_block_kernel): the guiding solution,
 // the outputs and a trace of the flipped indices (n entries of scratch).
 struct RelinkArgs {
@@ -600,101 +543,6 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
   }
 }
 
-// All passing starts of a batch of instances in one persistent launch, packed
-// by size.  Class c (0 .. 3) holds the instances whose n fits a sub-group of
-// T >> c threads (16 (T >> c) C elements; T >> 3 = 32 is one warp), and its
-// items form the range ranges[c] = {first item, items, 0, 0} (instances come
-// largest first, so each class is contiguous).  Each block runs the classes
-// in turn, split into 2^c sub-groups for class c, and every sub-group takes
-// the class's next start from its counter next[c] as soon as it has finished
-// the previous one: a block climbs up to eight small starts at once, and no
-// sub-group waits for another's longer climb except at the three class
-// boundaries.
-template <int T, int C, int R, int TS>
-__device__ __forceinline__ void climb_item(const BatchDesc* __restrict__ d, int2 it,
-                                           int32_t max_flips, int2* rec_flat,
-                                           uint4* spec_slots, int sg) {
-  const BatchDesc& b = d[it.x];
-  if (b.err[1] != 0) return;  // Q failed its symmetry check: no climb
-  const int s = b.idx[it.y];
-  if (s < 0 || s >= b.S) {
-    if ((int)threadIdx.x == sg * TS) atomicOr(b.err, UBQP_DEVERR_BADIDX);
-    return;
-  }
-  if constexpr (TS == T) {
-    Group<T> grp{reinterpret_cast<int2 (*)[T / 32]>(rec_flat), 0};
-    ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s, max_flips,
-                        b.flips ? b.flips + s : nullptr, b.err, spec_slots,
-                        b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
-  } else if constexpr (TS == 32) {  // one warp per start: warp-level reductions only
-    Group<32> grp;
-    ascend_one<32, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
-                         max_flips, b.flips ? b.flips + s : nullptr, b.err,
-                         spec_slots + sg * spec_slot_count<32, C, R>(),
-                         b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
-  } else {
-    SubGroup<TS> grp{reinterpret_cast<int2 (*)[TS / 32]>(rec_flat + sg * 2 * (TS / 32)), 0,
-                     sg * TS, 1 + sg};
-    ascend_one<TS, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
-                         max_flips, b.flips ? b.flips + s : nullptr, b.err,
-                         spec_slots + sg * spec_slot_count<TS, C, R>(),
-                         b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
-  }
-}
-
-// The sub-groups of one class take its starts: the first wave spread over the
-// blocks (start sg * blocks + block, so that a short list lands one start per
-// block, not several on the blocks of one SM), then from the class's counter
-// (or, without counters, round robin over all sub-groups of the grid).
-template <int T, int C, int R, int TS>
-__device__ __forceinline__ void climb_class(const BatchDesc* __restrict__ d,
-                                            const int2* __restrict__ items, int4 range,
-                                            int32_t max_flips, unsigned long long* next,
-                                            int2* rec_flat, uint4* spec_slots,
-                                            long long* slot) {
-  constexpr int K = T / TS;
-  const int sg = (int)threadIdx.x / TS, r = (int)threadIdx.x % TS;
-  auto sg_sync = [&]() {
-    if constexpr (TS == T) __syncthreads();
-    else if constexpr (TS == 32) __syncwarp();
-    else named_sync(1 + sg, TS);
-  };
-  const long long wave = (long long)gridDim.x * K;
-  for (long long k = 0;; ++k) {
-    long long t = (long long)sg * gridDim.x + blockIdx.x;
-    if (k > 0) {
-      if (r == 0) slot[sg] = next ? wave + (long long)atomicAdd(next, 1ull) : t + k * wave;
-      sg_sync();
-      t = slot[sg];
-      sg_sync();  // every thread has read slot[sg] before its leader writes it again
-    }
-    if (t >= range.y) break;
-    climb_item<T, C, R, TS>(d, items[range.x + t], max_flips, rec_flat, spec_slots, sg);
-  }
-}
-
-template <int T, int C, int R>
-__global__ void __launch_bounds__(T, 2)
-ascent_batch_packed_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ items,
-                           const int4* __restrict__ ranges, int32_t max_flips,
-                           unsigned long long* __restrict__ next) {
-  static_assert(T / 8 == 32, "sub-groups down to one warp");
-  __shared__ int2 rec_flat[2 * (T / 32)];
-  __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
-  __shared__ long long slot[8];
-  climb_class<T, C, R, T>(d, items, ranges[0], max_flips, next ? next : nullptr, rec_flat,
-                          spec_slots, slot);
-  __syncthreads();
-  climb_class<T, C, R, T / 2>(d, items, ranges[1], max_flips, next ? next + 1 : nullptr,
-                              rec_flat, spec_slots, slot);
-  __syncthreads();
-  climb_class<T, C, R, T / 4>(d, items, ranges[2], max_flips, next ? next + 2 : nullptr,
-                              rec_flat, spec_slots, slot);
-  __syncthreads();
-  climb_class<T, C, R, T / 8>(d, items, ranges[3], max_flips, next ? next + 3 : nullptr,
-                              rec_flat, spec_slots, slot);
-}
-
 // Independent warps, one start each (kWarps per block); counts, starts and
 // launch as in the block kernel, the first wave one warp per block over the
 // whole grid before any block's second warp.
@@ -733,6 +581,63 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                                     spec_slots + warp * spec_slot_count<32, C, R>(),
                                     Y ? Y + t * ldy : nullptr, grp, nullptr,
                                     TR ? trace + (int64_t)s * ldt : nullptr, ldt);
+  }
+}
+
+// The passing starts of one size class of a batch (launch_ascent_batch_packed):
+// items[ranges[cls].x .. + ranges[cls].y), every instance with n <= 16 T C, T
+// threads per start (T = 32: kWarps starts per block).  First wave and counter
+// as in the kernels above.  Climbs only when the batch's total number of items
+// lies in [lo, hi].
+template <int T, int C, int R, int OCC>
+__global__ void __launch_bounds__(T == 32 ? 32 * kWarps : T, OCC)
+ascent_class_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ items,
+                    const int4* __restrict__ ranges, int cls,
+                    const int64_t* __restrict__ n_items, int32_t max_flips,
+                    unsigned long long* __restrict__ next, int64_t lo, int64_t hi) {
+  constexpr int PER = T == 32 ? kWarps : 1;
+  __shared__ int2 rec[2][T / 32];
+  __shared__ uint4 spec_slots[PER * spec_slot_count<T, C, R>()];
+  __shared__ unsigned long long ticket;
+  const int64_t total = *n_items;
+  if (total < lo || total > hi) return;
+  const int4 range = ranges[cls];
+  const int sub = (int)threadIdx.x / T, rank = (int)threadIdx.x % T;
+  const int64_t wave = (int64_t)gridDim.x * PER;
+  for (int64_t t = (int64_t)sub * gridDim.x + blockIdx.x; t < range.y;) {
+    const int2 it = items[range.x + t];
+    const BatchDesc& b = d[it.x];
+    const int s = b.idx[it.y];
+    if (b.err[1] == 0) {  // else Q failed its symmetry check: no climb
+      if (s < 0 || s >= b.S) {
+        if (rank == 0) atomicOr(b.err, UBQP_DEVERR_BADIDX);
+      } else {
+        const float* y = b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr;
+        int32_t* fl = b.flips ? b.flips + s : nullptr;
+        if constexpr (T == 32) {
+          Group<32> grp;
+          ascend_one<32, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
+                               max_flips, fl, b.err,
+                               spec_slots + sub * spec_slot_count<32, C, R>(), y, grp);
+        } else {
+          Group<T> grp{rec, 0};
+          ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
+                              max_flips, fl, b.err, spec_slots, y, grp);
+        }
+      }
+    }
+    if (!next) {
+      t += wave;
+    } else if constexpr (T == 32) {
+      unsigned long long v = 0;
+      if (rank == 0) v = atomicAdd(&next[cls], 1ull);
+      t = wave + (int64_t)__shfl_sync(0xffffffffu, v, 0);
+    } else {
+      __syncthreads();  // rec is free for the next start; ticket was read
+      if (rank == 0) ticket = atomicAdd(&next[cls], 1ull);
+      __syncthreads();
+      t = wave + (int64_t)ticket;
+    }
   }
 }
 
@@ -936,6 +841,18 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
     return tiers(UBQP_C(256, 2, 1, 1), UBQP_C(256, 2, 1, 2), UBQP_C(128, 4, 0, 3), full);
   return UBQP_C(512, 2, 1, 1).launch(a, 0, INT64_MAX);
 #undef UBQP_C
+}
+
+template <int T, int C, int R, int OCC>
+cudaError_t launch_class(const BatchDesc* d, const int2* items, const int4* ranges, int cls,
+                         const int64_t* n_items, int32_t max_flips, unsigned long long* next,
+                         int64_t most, int64_t lo, int64_t hi, int sm_count, cudaStream_t st) {
+  constexpr int kBlock = T == 32 ? 32 * kWarps : T, kPer = kBlock / T;
+  int64_t grid = resident_grid(ascent_class_kernel<T, C, R, OCC>, kBlock, sm_count);
+  if (grid > (most + kPer - 1) / kPer) grid = (most + kPer - 1) / kPer;
+  ascent_class_kernel<T, C, R, OCC><<<(unsigned)grid, kBlock, 0, st>>>(
+      d, items, ranges, cls, n_items, max_flips, next, lo, hi);
+  return cudaGetLastError();
 }
 
 template <int T, int C>

@@ -61,42 +61,33 @@ __global__ void __launch_bounds__(THREADS) best_batch_kernel(const BatchDesc* __
 // every passing start, instances in the given order (largest first).
 // The instances order[k0 .. k0 + m) (m <= THREADS) of a batch's lists: each
 // thread reads one instance's passing count (and, for the packed list, its
-// unit class), then one thread turns them into exclusive offsets in shared
-// memory, so that no global load waits inside the loop over instances.  With
-// skip0 the instances of class 0 (climbed by launches of their own) add no
-// items.
+// class), then one thread turns them into exclusive offsets in shared memory,
+// so that no global load waits inside the loop over instances.  In the packed
+// list the instances above the last class (climbed by launches of their own)
+// add no items.
 struct ListChunk {
   int inst[THREADS];
   int cls[THREADS];
-  long long cnt[THREADS], base[THREADS], ubase[THREADS];
-  long long base_end, ubase_end;
+  long long cnt[THREADS], base[THREADS];
+  long long base_end;
 };
 __device__ void list_chunk(const BatchDesc* __restrict__ d, const int32_t* __restrict__ order,
-                           int k0, int m, int T, int C, bool packed, bool skip0, ListChunk& L) {
+                           int k0, int m, bool packed, ListChunk& L) {
   if ((int)threadIdx.x < m) {
     const int i = order[k0 + (int)threadIdx.x];
     const int n = d[i].n;
     L.inst[threadIdx.x] = i;
-    L.cnt[threadIdx.x] = *d[i].count;
-    L.cls[threadIdx.x] = !packed                 ? 0
-                         : n <= 16 * (T >> 3) * C ? 3
-                         : n <= 16 * (T >> 2) * C ? 2
-                         : n <= 16 * (T >> 1) * C ? 1
-                                                  : 0;
-    if (skip0 && L.cls[threadIdx.x] == 0) L.cnt[threadIdx.x] = 0;
+    L.cls[threadIdx.x] = packed_class(n);
+    L.cnt[threadIdx.x] = packed && packed_own_climb(n) ? 0 : *d[i].count;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    long long b = L.base_end, ub = L.ubase_end;
+    long long b = L.base_end;
     for (int j = 0; j < m; ++j) {
       L.base[j] = b;
-      L.ubase[j] = ub;
-      const long long per = 1ll << L.cls[j];
       b += L.cnt[j];
-      ub += (L.cnt[j] + per - 1) / per;
     }
     L.base_end = b;
-    L.ubase_end = ub;
   }
   __syncthreads();
 }
@@ -105,10 +96,10 @@ __global__ void __launch_bounds__(THREADS)
 batch_items_kernel(const BatchDesc* __restrict__ d, const int32_t* __restrict__ order, int count,
                    int2* __restrict__ items, int64_t* __restrict__ n_items) {
   __shared__ ListChunk L;
-  if (threadIdx.x == 0) L.base_end = L.ubase_end = 0;
+  if (threadIdx.x == 0) L.base_end = 0;
   for (int k0 = 0; k0 < count; k0 += THREADS) {
     const int m = count - k0 < THREADS ? count - k0 : THREADS;
-    list_chunk(d, order, k0, m, 0, 0, false, false, L);
+    list_chunk(d, order, k0, m, false, L);
     for (int j = 0; j < m; ++j)
       for (long long t = threadIdx.x; t < L.cnt[j]; t += THREADS)
         items[L.base[j] + t] = make_int2(L.inst[j], (int)t);
@@ -118,24 +109,21 @@ batch_items_kernel(const BatchDesc* __restrict__ d, const int32_t* __restrict__ 
 }
 
 // The work list of the packed batch ascent: the items as batch_items_kernel
-// writes them, and the range {first item, items, 0, 0} of each class c = 0 ..
-// 3, an instance being of the largest class whose sub-group of T >> c threads
-// (16 (T >> c) C elements) holds its n.  Instances come largest first, so
-// each class's items are contiguous.  With skip0 class 0 is left out (its
-// instances climb in launches of their own).
+// writes them, and the range {first item, items, 0, 0} of each class.
+// Instances come largest first, so each class's items are contiguous.
 __global__ void __launch_bounds__(THREADS)
 batch_units_kernel(const BatchDesc* __restrict__ d, const int32_t* __restrict__ order, int count,
-                   int T, int C, int skip0, int2* __restrict__ items, int4* __restrict__ ranges,
+                   int2* __restrict__ items, int4* __restrict__ ranges,
                    int64_t* __restrict__ n_items) {
   __shared__ ListChunk L;
-  __shared__ long long cbeg[4], ccnt[4];
+  __shared__ long long cbeg[kPackedClasses], ccnt[kPackedClasses];
   if (threadIdx.x == 0) {
-    L.base_end = L.ubase_end = 0;
-    for (int c = 0; c < 4; ++c) cbeg[c] = -1, ccnt[c] = 0;
+    L.base_end = 0;
+    for (int c = 0; c < kPackedClasses; ++c) cbeg[c] = -1, ccnt[c] = 0;
   }
   for (int k0 = 0; k0 < count; k0 += THREADS) {
     const int m = count - k0 < THREADS ? count - k0 : THREADS;
-    list_chunk(d, order, k0, m, T, C, true, skip0 != 0, L);
+    list_chunk(d, order, k0, m, true, L);
     if (threadIdx.x == 0)
       for (int j = 0; j < m; ++j) {
         const int c = L.cls[j];
@@ -148,7 +136,7 @@ batch_units_kernel(const BatchDesc* __restrict__ d, const int32_t* __restrict__ 
     __syncthreads();  // L is rewritten by the next chunk
   }
   if (threadIdx.x == 0) {
-    for (int c = 0; c < 4; ++c)
+    for (int c = 0; c < kPackedClasses; ++c)
       ranges[c] = make_int4(cbeg[c] < 0 ? 0 : (int)cbeg[c], (int)ccnt[c], 0, 0);
     *n_items = L.base_end;
   }
@@ -308,11 +296,9 @@ cudaError_t launch_batch_items(const BatchDesc* d, const int32_t* order, int cou
   return cudaGetLastError();
 }
 
-cudaError_t launch_batch_units(const BatchDesc* d, const int32_t* order, int count, int T, int C,
-                               bool skip0, int2* items, int4* ranges, int64_t* n_items,
-                               cudaStream_t st) {
-  batch_units_kernel<<<1, THREADS, 0, st>>>(d, order, count, T, C, skip0 ? 1 : 0, items, ranges,
-                                            n_items);
+cudaError_t launch_batch_units(const BatchDesc* d, const int32_t* order, int count, int2* items,
+                               int4* ranges, int64_t* n_items, cudaStream_t st) {
+  batch_units_kernel<<<1, THREADS, 0, st>>>(d, order, count, items, ranges, n_items);
   return cudaGetLastError();
 }
 

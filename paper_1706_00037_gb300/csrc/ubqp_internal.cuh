@@ -301,25 +301,35 @@ cudaError_t launch_batch_items(const BatchDesc* d, const int32_t* order, int cou
 cudaError_t launch_ascent_batch(const BatchDesc* d, const int2* items, const int64_t* n_items,
                                 int T, int C, int32_t max_flips, int grid,
                                 unsigned long long* next, cudaStream_t st);
-// packed batch ascent: blocks of T threads split into sub-groups of T, T/2,
-// T/4 or T/8 threads by n; the items of each of the four classes form one
-// range (ranges: 4 int4 {first item, items, 0, 0}; n_items: the item count),
-// and next holds one start counter per class (4 x 8 bytes, zeroed by the
-// launch; NULL: round robin).  skip0: class 0 left out of the list (its
-// instances climbed by launch_ascent of their own; see packed_own_climb)
-cudaError_t launch_batch_units(const BatchDesc* d, const int32_t* order, int count, int T, int C,
-                               bool skip0, int2* items, int4* ranges, int64_t* n_items,
-                               cudaStream_t st);
-// Packed batch climbs leave the instances too large for half a block (class
-// 0) to the single-instance launcher, whose group shapes for large n climb
-// faster (n = 5000, ~450 passers: 1.40 ms with 160-thread groups three per SM
-// against 2.01 ms packed).
-inline bool packed_own_climb(int n, int T, int C) { return n > 16 * (T / 2) * C; }
+// Packed batch ascent: the instances fall into classes by n, class c holding
+// packed_max_n(c - 1) < n <= packed_max_n(c), and each class is climbed by a
+// launch of its own (launch_ascent_batch_packed), whose group shape fits its
+// n.  Larger instances are left out of the list and climbed one launch per
+// instance (launch_ascent): their own shapes per count are worth more than a
+// shared launch (n = 5000, ~450 passers: 1.40 against 2.01 ms).
+constexpr int kPackedClasses = 6;
+__host__ __device__ constexpr int packed_max_n(int c) { return c < 4 ? 512 * (c + 1) : 1024 * (c - 1); }
+__host__ __device__ inline bool packed_own_climb(int n) {
+  return n > packed_max_n(kPackedClasses - 1);
+}
+__host__ __device__ inline int packed_class(int n) {
+  int c = 0;
+  while (c < kPackedClasses - 1 && n > packed_max_n(c)) ++c;
+  return c;
+}
+// The items of the packed list (instances largest first, those above the last
+// class left out), the range {first item, items, 0, 0} of each class, and the
+// item count.
+cudaError_t launch_batch_units(const BatchDesc* d, const int32_t* order, int count, int2* items,
+                               int4* ranges, int64_t* n_items, cudaStream_t st);
+// The climb of class cls; next: one start counter per class, zero at launch
+// (NULL: round robin).  most / batch_most: the most items the class / the
+// batch can have.
 cudaError_t launch_ascent_batch_packed(const BatchDesc* d, const int2* items, const int4* ranges,
-                                       int T, int C, int32_t max_flips, int grid,
+                                       int cls, const int64_t* n_items, int64_t most,
+                                       int64_t batch_most, int32_t max_flips, int sm_count,
                                        unsigned long long* next, cudaStream_t st);
 bool ascent_packed_supported(int T, int C);
-int ascent_packed_grid(int T, int C, int sm_count);
 int ascent_batch_grid(int T, int C, int sm_count);
 bool ascent_batch_supported(int T, int C);
 cudaError_t launch_best_batch(const BatchDesc* d, int count, cudaStream_t st);

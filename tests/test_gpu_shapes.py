@@ -80,3 +80,19 @@ def test_relink_shapes_agree(n):
         xb, fb, d, *_ = orc.relink1(Q, Xh[p], Gh[p])
         assert (int(got[1][p]), int(got[2][p])) == (fb, d)
         assert np.array_equal(got[0][p].cpu().numpy().view(np.uint64), xb)
+
+
+@pytest.mark.parametrize("S", [64, 400])
+def test_packed_classes_equal_single_solves(S):
+    """The packed batch climb at the edges of its size classes, with few starts
+    in all and with more than ten per SM."""
+    insts = [ubqp.Instance(torch.from_numpy(instance(n, "small")).cuda())
+             for n in (512, 513, 1024, 1025, 1536, 1537, 2048, 2049, 3072, 3073, 4096, 4097)]
+    p = ubqp.make_params(S, 0.25, seed=5)
+    batch = ubqp.Batch(insts, p)
+    batch.set(256, 2, packed=True)
+    batch.run(5)
+    for i, inst in enumerate(insts):
+        bx, bf = batch.result(i)
+        x, f, _ = ubqp.solve(inst, p, want_stats=False)
+        assert torch.equal(bx, x) and torch.equal(bf, f), inst.n
