@@ -16,6 +16,8 @@ constexpr int64_t kTimeoutNs = 20ll * 1000 * 1000 * 1000;  // per start
 // (passing starts of 1000 random ones): one row is 3-13% faster than none;
 // two or more cost more in reductions and copies than their hits save.
 constexpr int kSpecRows = 1;
+// Starts per block of the one-warp kernels.
+constexpr int kWarps = 2;
 // shared-memory slots (16 bytes each) of a group of T threads: two buffers of
 // R rows x C chunks per thread, laid out thread-minor
 template <int T, int C, int R>
@@ -66,20 +68,19 @@ constexpr int kOutKey = -(1 << 30);
 // index (about log2(E) branches instead of E predicated operations): its key
 // becomes that of the gain -gain (relinking: it leaves the candidates) with
 // the element's own term of the row update that follows, -2 q_kk, taken off
-// beforehand, and its selector changes sign.
+// beforehand; its selector changes sign and its x bit flips.  q_kk comes from
+// shared memory, not from the row, so the flip does not wait for the row.
 template <int LO, int HI, int E, bool RL>
 __device__ __forceinline__ void flip_tree(int (&key)[E], uint32_t (&sel)[E],
-                                          uint32_t (&xm)[(E + 31) / 32],
-                                          const int (&q)[E / 4], int ek, int gain) {
+                                          uint32_t (&xm)[(E + 31) / 32], int ek, int v) {
   if constexpr (HI - LO == 1) {
-    const int qkk = (int)(int8_t)((unsigned)q[LO >> 2] >> (8 * (LO & 3)));
-    key[LO] = RL ? kOutKey : ((2 * qkk - gain) << kKeyBits) + (31 - (LO & 31));
+    key[LO] = RL ? kOutKey : v + (31 - (LO & 31));
     sel[LO] ^= 0x80u << (8 * (LO & 3));
     xm[LO >> 5] ^= 1u << (LO & 31);
   } else {
     constexpr int MID = (LO + HI) / 2;
-    if (ek < MID) flip_tree<LO, MID, E, RL>(key, sel, xm, q, ek, gain);
-    else flip_tree<MID, HI, E, RL>(key, sel, xm, q, ek, gain);
+    if (ek < MID) flip_tree<LO, MID, E, RL>(key, sel, xm, ek, v);
+    else flip_tree<MID, HI, E, RL>(key, sel, xm, ek, v);
   }
 }
 
@@ -172,6 +173,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
                                            int64_t* __restrict__ f_s, int32_t max_flips,
                                            int32_t* __restrict__ flips_s,
                                            unsigned* __restrict__ err, uint4* spec_slots,
+                                           uint4* diag,
                                            const float* __restrict__ y_g, G& grp,
                                            const RelinkArgs* rl = nullptr,
                                            uint16_t* __restrict__ trace_row = nullptr,
@@ -220,6 +222,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     for (int v = 0; v < 4; ++v)
       y4[v] = y_g && j0 < ldy ? reinterpret_cast<const float4*>(y_g + j0)[v]
                               : make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t dg[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int o = 0; o < 16; ++o) {
       const int e = c * 16 + o, j = j0 + o;
@@ -230,7 +233,9 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       const int qjj = cd ? Q8[(int64_t)j * ldq + j] : 0;
       key[e] = cd ? ((qjj + (xb ? -y2 : y2)) << kKeyBits) + (31 - (e & 31)) : kOutKey;
       sel[e] = (xb ? 0xC0u : 0x40u) << (8 * (o & 3));
+      dg[o >> 2] |= (uint32_t)(uint8_t)qjj << (8 * (o & 3));
     }
+    diag[c * T + g] = make_uint4(dg[0], dg[1], dg[2], dg[3]);  // read by this thread only
   }
   for (int w = 0; w < W && !y_g; ++w) {
     uint64_t word = x_g[w] & valid_mask(n, w);
@@ -318,32 +323,12 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   int64_t fbest = fval;
   int tbest = 0;
   const uint64_t t0 = globaltimer();
+  const int last = RL ? dist - 1 : max_flips;  // relinking: the last step only reaches g
+  int lim = min(last, 1023);                   // the next move count to look at
   for (;;) {
-    if (RL) {
-      if (flips >= dist - 1) break;  // the last step only reaches g
-    } else {
-      if (best.x <= 0 || flips >= max_flips) break;
-    }
-    if ((flips & 1023) == 1023) {
-      const bool late = (int64_t)(globaltimer() - t0) > kTimeoutNs;
-      if (grp.any(late)) {
-        if (g == 0) atomicOr(err, UBQP_DEVERR_TIMEOUT);
-        break;
-      }
-    }
-    const int k = best.y >> 1;
-    fval += best.x;
-    ++flips;
-    if (RL) {
-      if (flips < dist && (tbest == 0 || fval > fbest)) {
-        fbest = fval;
-        tbest = flips;
-      }
-      if (g == 0) rl->trace[flips - 1] = (uint16_t)k;
-    }
-    if constexpr (TR) {  // the move record: flipped indices in order
-      if (g == 0 && flips <= trace_cap) trace_row[flips - 1] = (uint16_t)k;
-    }
+    // the row first: everything up to the update runs in the shadow of its
+    // load (a load for the move that is not made reads a valid row)
+    const int k = RL ? min(best.y >> 1, n - 1) : best.y >> 1;
     int q[4 * C];
     bool hit = false;
     if constexpr (R > 0) {
@@ -373,6 +358,27 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
         q[4 * c + 3] = (int)v.w;
       }
     }
+    if ((!RL && best.x <= 0) || flips >= lim) {
+      if ((!RL && best.x <= 0) || flips >= last) break;
+      const bool late = (int64_t)(globaltimer() - t0) > kTimeoutNs;
+      if (grp.any(late)) {
+        if (g == 0) atomicOr(err, UBQP_DEVERR_TIMEOUT);
+        break;
+      }
+      lim = min(last, flips + 1024);
+    }
+    fval += best.x;
+    ++flips;
+    if (RL) {
+      if (flips < dist && (tbest == 0 || fval > fbest)) {
+        fbest = fval;
+        tbest = flips;
+      }
+      if (g == 0) rl->trace[flips - 1] = (uint16_t)k;
+    }
+    if constexpr (TR) {  // the move record: flipped indices in order
+      if (g == 0 && flips <= trace_cap) trace_row[flips - 1] = (uint16_t)k;
+    }
     if constexpr (R > 0) {  // fetch the runners-up's rows for the next move
       grp.template runners<R>(best.y, cand);
       // the copies into this buffer two moves ago have landed
@@ -381,15 +387,13 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       for (int i = 0; i < R; ++i) {
         const int r = cand[i] >> 1;
         prow[i] = r < n ? r : -1;
+        const int from = r < n ? r : 0;
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-          if (prow[i] >= 0) {
-            const uint4* src = row_chunk(prow[i], c);
-            const uint32_t a = slot0 + (uint32_t)((buf * RR + i) * C + c) * (T * 16);
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(a), "l"(src)
-                         : "memory");
-          }
-        }
+        for (int c = 0; c < C; ++c)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                           slot0 + (uint32_t)((buf * RR + i) * C + c) * (T * 16)),
+                       "l"(row_chunk(from, c))
+                       : "memory");
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
       buf ^= 1;
@@ -406,8 +410,9 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     // the owner of k flips x_k (when relinking, k leaves the candidates)
     const int kc = k / CW, kr = k - kc * CW;
     if ((kr >> 4) == g) {
-      const int ek = kc * 16 + (kr & 15);
-      flip_tree<0, E, E, RL>(key, sel, xm, q, ek, best.x);
+      const int qkk = reinterpret_cast<const int8_t*>(diag)[k];
+      flip_tree<0, E, E, RL>(key, sel, xm, kc * 16 + (kr & 15),
+                                (2 * qkk - best.x) * (1 << kKeyBits));
     }
 #pragma unroll
     for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = INT_MIN;
@@ -477,6 +482,7 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                     int64_t ldt, int64_t cnt_lo, int64_t cnt_hi) {
   __shared__ int2 rec[2][T / 32];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
+  __shared__ uint4 diag[T * C];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
   pdl_wait();  // no early release: see pdl_release
@@ -499,7 +505,7 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
       continue;
     }
     ascend_one<T, C, R, false, TR>(Q8, ldq, ldy, n, W, X + (int64_t)s * W, f + s, max_flips,
-                                   flips ? flips + s : nullptr, err, spec_slots,
+                                   flips ? flips + s : nullptr, err, spec_slots, diag,
                                    Y ? Y + t * ldy : nullptr, grp, nullptr,
                                    TR ? trace + (int64_t)s * ldt : nullptr, ldt);
   }
@@ -514,6 +520,7 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
                     unsigned long long* __restrict__ next) {
   __shared__ int2 rec[2][T / 32];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
+  __shared__ uint4 diag[T * C];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
   const int64_t cnt = *n_items;
@@ -537,8 +544,9 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
       if (threadIdx.x == 0) atomicOr(b.err, UBQP_DEVERR_BADIDX);
       continue;
     }
-    ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s, max_flips,
-                     b.flips ? b.flips + s : nullptr, b.err, spec_slots,
+    ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W,
+                     b.X + (int64_t)s * b.W, b.f + s, max_flips,
+                     b.flips ? b.flips + s : nullptr, b.err, spec_slots, diag,
                      b.Y ? b.Y + (int64_t)it.y * b.ldy : nullptr, grp);
   }
 }
@@ -546,7 +554,6 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
 // Independent warps, one start each (kWarps per block); counts, starts and
 // launch as in the block kernel, the first wave one warp per block over the
 // whole grid before any block's second warp.
-constexpr int kWarps = 2;
 template <int C, int R, bool TR, int OCC>
 __global__ void __launch_bounds__(32 * kWarps, OCC)
 ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
@@ -557,6 +564,7 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                    unsigned long long* __restrict__ next, uint16_t* __restrict__ trace,
                    int64_t ldt, int64_t cnt_lo, int64_t cnt_hi) {
   __shared__ uint4 spec_slots[kWarps * spec_slot_count<32, C, R>()];
+  __shared__ uint4 diag[kWarps * 32 * C];
   Group<32> grp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait();  // no early release: see pdl_release
@@ -579,6 +587,7 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
     ascend_one<32, C, R, false, TR>(Q8, ldq, ldy, n, W, X + (int64_t)s * W, f + s, max_flips,
                                     flips ? flips + s : nullptr, err,
                                     spec_slots + warp * spec_slot_count<32, C, R>(),
+                                    diag + warp * (32 * C),
                                     Y ? Y + t * ldy : nullptr, grp, nullptr,
                                     TR ? trace + (int64_t)s * ldt : nullptr, ldt);
   }
@@ -598,6 +607,7 @@ ascent_class_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
   constexpr int PER = T == 32 ? kWarps : 1;
   __shared__ int2 rec[2][T / 32];
   __shared__ uint4 spec_slots[PER * spec_slot_count<T, C, R>()];
+  __shared__ uint4 diag[PER * T * C];
   __shared__ unsigned long long ticket;
   const int64_t total = *n_items;
   if (total < lo || total > hi) return;
@@ -618,11 +628,13 @@ ascent_class_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
           Group<32> grp;
           ascend_one<32, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
                                max_flips, fl, b.err,
-                               spec_slots + sub * spec_slot_count<32, C, R>(), y, grp);
+                               spec_slots + sub * spec_slot_count<32, C, R>(),
+                               diag + sub * (32 * C), y, grp);
         } else {
           Group<T> grp{rec, 0};
-          ascend_one<T, C, R>(b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s,
-                              max_flips, fl, b.err, spec_slots, y, grp);
+          ascend_one<T, C, R>(
+              b.Q8, b.ldq, b.ldy, b.n, b.W, b.X + (int64_t)s * b.W, b.f + s, max_flips, fl, b.err,
+              spec_slots, diag, y, grp);
         }
       }
     }
@@ -657,6 +669,7 @@ relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
   __shared__ int2 rec[2][T / 32];
   __shared__ uint64_t xs[UBQP_MAX_N / 64];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
+  __shared__ uint4 diag[T * C];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
   if (err[1] != 0) return;  // Q failed its symmetry check: no walk
@@ -676,7 +689,7 @@ relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                        trace + p * ldt, xs};
     int64_t f0 = f[p];
     ascend_one<T, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
-                              nullptr, err, spec_slots, Y ? Y + p * ldy : nullptr, grp, &a);
+                              nullptr, err, spec_slots, diag, Y ? Y + p * ldy : nullptr, grp, &a);
   }
 }
 
@@ -691,6 +704,7 @@ relink_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                    unsigned long long* __restrict__ next) {
   __shared__ uint64_t xs_all[4][16];
   __shared__ uint4 spec_slots[4 * spec_slot_count<32, C, R>()];
+  __shared__ uint4 diag[4 * 32 * C];
   Group<32> grp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (err[1] != 0) return;  // Q failed its symmetry check: no walk
@@ -708,6 +722,7 @@ relink_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
     ascend_one<32, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
                                nullptr, err,
                                spec_slots + warp * spec_slot_count<32, C, R>(),
+                               diag + warp * (32 * C),
                                Y ? Y + p * ldy : nullptr, grp, &a);
   }
 }
@@ -784,11 +799,11 @@ struct Climb {
 //        copies, for lists that keep every SM busy: there the issue slots
 //        bound the climb, and the copies cost more than their hits save.
 // Measured on 1000 to 12 000 diversified starts, the passing ones climbed (us,
-// before -> now): n = 1025, 510 starts 187 -> 143; 2500, 542 starts 533 -> 359;
-// 1000, 5638 starts 784 -> 411; 1400, 6069: 1382 -> 701; 2000, 4214: 1406 ->
-// 967; 2500, 3213: 2082 -> 1343; 4000, 2193: 3046 -> 2091; 5000, 4469: 9080 ->
-// 5433; 6000, 2187: 7464 -> 3727; 7000, 54: 1857 -> 1697; 7000, 641: 3364 ->
-// 2663; 7000, 2172: 9610 -> 6535.  The boundary between mid and all lies where
+// with y, S, C registers -> now): n = 1025, 510 starts 187 -> 136; 2500, 542
+// starts 533 -> 353; 1000, 5638 starts 784 -> 359; 1400, 6069: 1382 -> 677;
+// 2000, 4214: 1406 -> 853; 2500, 3213: 2082 -> 1152; 4000, 2193: 3046 -> 1833;
+// 5000, 4469: 9080 -> 5369; 6000, 2187: 7464 -> 3655; 7000, 54: 1857 -> 1636;
+// 7000, 641: 3364 -> 2606; 7000, 2172: 9610 -> 5243.  The boundary between mid and all lies where
 // a list of that n keeps mid's SMs busy anyway: both take the same time near
 // 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000 starts 2178
 // and 2077), earlier where mid fits only two or three blocks (n = 4800, 600

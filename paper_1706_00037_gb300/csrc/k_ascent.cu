@@ -25,18 +25,23 @@
 // threads keep one maximum per 32); across threads the group reduces (gain,
 // 2j + x) with warp max/min reductions (redux.sync), so every thread learns k,
 // x_k and Delta_k.  The thread owning k resets key_k to -Delta_k, turns sel_k
-// and flips its x bit.  Rows are read from L2 (the int8 Q of one instance,
+// and flips its x bit; it takes q_kk from a copy of the diagonal in shared
+// memory, so that nothing but the update itself waits for the row (with q_kk
+// taken from the row the owner's branches came after the load: n = 7000, 2172
+// starts 6.53 -> 5.24 ms, 54 starts 1.70 -> 1.64).  Rows are read from L2 (the int8 Q of one instance,
 // e.g. 49 MB at n = 7000, stays resident there); nothing per move goes to HBM.
 //
 // What bounds it.  With few starts the chain of moves is latency-bound: per
 // move a dependent L2 row fetch, the update and a block-wide reduction (n =
-// 7000, 54 starts: 791 cycles per move, 1.70 ms; 863 and 1.85 before).  The
-// fetch is taken off the chain when the move was predicted: every move also
+// 7000, 54 starts: 763 cycles per move, 1.64 ms; 863 and 1.85 with y, S and C
+// registers).  The loads of the row are issued before anything else of the
+// move, its end test included; the runner-up reduction, the selectors' flip and
+// the owner's branches run in their shadow.  The fetch is taken off the chain when the move was predicted: every move also
 // copies the row of the reduction's runner-up into shared memory, and the next
 // move is that row often enough (about 40% at n = 7000) to pay for the copies.
-// With many starts the issue slots bound it (n = 1400, 6069 starts: 190 warp
-// instructions per move, 101 cycles per move and SM, 0.70 ms; 199 cycles and
-// 1.38 ms before).  launch_ascent_shaped picks the group shape by n and count.
+// With many starts the issue slots and the latency of 12 to 20 warps bound it
+// (n = 1400, 6069 starts: about 185 warp instructions per move, 97 cycles per
+// move and SM, 0.68 ms; 199 cycles and 1.38 ms with y, S and C registers).  launch_ascent_shaped picks the group shape by n and count.
 //
 // Start-up: y = Q x of every listed start comes from the tensor-core product of
 // the ascent workspace when given (exact integers in fp32), else each group
