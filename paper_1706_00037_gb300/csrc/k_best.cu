@@ -10,6 +10,7 @@ namespace {
 
 constexpr int THREADS = 1024;
 constexpr int WARPS = THREADS / 32;
+static_assert(WARPS == 32, "the block-wide steps read one warp's partial per lane");
 
 __device__ void block_best(const int64_t* __restrict__ f, const uint64_t* __restrict__ X,
                            int64_t S, int W, uint64_t* __restrict__ best_x,
@@ -22,21 +23,17 @@ __device__ void block_best(const int64_t* __restrict__ f, const uint64_t* __rest
     long long v = f[b];
     if (v > mx) { mx = v; am = b; }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    long long om = __shfl_xor_sync(0xffffffffu, mx, o);
-    long long oa = __shfl_xor_sync(0xffffffffu, am, o);
-    if (om > mx || (om == mx && oa < am)) { mx = om; am = oa; }
-  }
+  warp_max64(mx, am);
   if (lane == 0) { s_max[warp] = mx; s_arg[warp] = am; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long m = LLONG_MIN, a = LLONG_MAX;
-    for (int i = 0; i < WARPS; ++i)
-      if (s_max[i] > m || (s_max[i] == m && s_arg[i] < a)) { m = s_max[i]; a = s_arg[i]; }
-    best_f[0] = m;
-    best_f[1] = a;
-    s_best = a;
+  if (warp == 0) {
+    long long m = s_max[lane], a = s_arg[lane];
+    warp_max64(m, a);
+    if (lane == 0) {
+      best_f[0] = m;
+      best_f[1] = a;
+      s_best = a;
+    }
   }
   __syncthreads();
   const long long a = s_best;
@@ -184,26 +181,24 @@ __device__ void block_solve_stats(const int64_t* __restrict__ count,
     tot += v;
     mx = v > mx ? v : mx;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    long long v = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = v > mx ? v : mx;
-  }
+  long long none = 0;
+  tot = warp_sum64(tot);
+  warp_max64(mx, none);
   if (lane == 0) { s_tot[warp] = tot; s_mx[warp] = mx; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long t = 0, m = 0;
-    for (int i = 0; i < WARPS; ++i) {
-      t += s_tot[i];
-      m = s_mx[i] > m ? s_mx[i] : m;
+  if (warp == 0) {
+    long long t = s_tot[lane], m = s_mx[lane];
+    none = 0;
+    t = warp_sum64(t);
+    warp_max64(m, none);
+    if (lane == 0) {
+      out[0] = c;
+      out[1] = t;
+      out[2] = m;
+      out[3] = sstats[1];
+      out[4] = best[1];
+      out[5] = sstats[0];
     }
-    out[0] = c;
-    out[1] = t;
-    out[2] = m;
-    out[3] = sstats[1];
-    out[4] = best[1];
-    out[5] = sstats[0];
   }
 }
 
@@ -249,18 +244,18 @@ search_update_kernel(const int64_t* __restrict__ f, const uint64_t* __restrict__
   const int64_t c = *count;
   long long tot = 0;
   for (int64_t t = threadIdx.x; t < c; t += THREADS) tot += flips[idx[t]];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  tot = warp_sum64(tot);
   if (lane == 0) s_tot[warp] = tot;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long t = 0;
-    for (int i = 0; i < WARPS; ++i) t += s_tot[i];
-    stats[0] += c;
-    stats[1] += t;
-    s_take = cand[0] > inc_f[0];
-    if (s_take) inc_f[0] = cand[0];
-    *history = inc_f[0];
+  if (warp == 0) {
+    const long long t = warp_sum64(s_tot[lane]);
+    if (lane == 0) {
+      stats[0] += c;
+      stats[1] += t;
+      s_take = cand[0] > inc_f[0];
+      if (s_take) inc_f[0] = cand[0];
+      *history = inc_f[0];
+    }
   }
   __syncthreads();
   if (s_take)

@@ -1,7 +1,7 @@
 // k_screen.cu -- the screen of the Pseudocode section: T(lambda) = Mean +
 // lambda (Max - Mean) over the batch, then the stable list of indices with
 // f_b > T (Fig. 2).  Two single-block kernels: the statistics (an exact int64
-// sum and a max with its lowest index, by warp shuffles), and the threshold in
+// sum and a max with its lowest index, by warp reductions), and the threshold in
 // double with explicitly rounded operations (no FMA) followed by a block-wide
 // ballot/prefix-sum compaction.  One launch runs both for a whole batch; the
 // split launches let a batch sharded over ranks combine the statistics before
@@ -15,6 +15,7 @@ namespace {
 
 constexpr int THREADS = 1024;
 constexpr int WARPS = THREADS / 32;
+static_assert(WARPS == 32, "the block-wide steps read one warp's partial per lane");
 
 // stats = {sum of f, max f, lowest index attaining it + offset}; one block.
 __device__ void block_screen_stats(const int64_t* __restrict__ f, int64_t S, int64_t offset,
@@ -29,24 +30,19 @@ __device__ void block_screen_stats(const int64_t* __restrict__ f, int64_t S, int
     sum += v;
     if (v > mx) { mx = v; am = b; }  // increasing b per thread: keeps lowest
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    long long om = __shfl_xor_sync(0xffffffffu, mx, o);
-    long long oa = __shfl_xor_sync(0xffffffffu, am, o);
-    if (om > mx || (om == mx && oa < am)) { mx = om; am = oa; }
-  }
+  sum = warp_sum64(sum);
+  warp_max64(mx, am);
   if (lane == 0) { s_sum[warp] = sum; s_max[warp] = mx; s_arg[warp] = am; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    long long t = 0, m = LLONG_MIN, a = LLONG_MAX;
-    for (int i = 0; i < WARPS; ++i) {
-      t += s_sum[i];
-      if (s_max[i] > m || (s_max[i] == m && s_arg[i] < a)) { m = s_max[i]; a = s_arg[i]; }
+  if (warp == 0) {  // WARPS == 32: one partial per lane
+    long long t = s_sum[lane], m = s_max[lane], a = s_arg[lane];
+    t = warp_sum64(t);
+    warp_max64(m, a);
+    if (lane == 0) {
+      stats[0] = t;
+      stats[1] = m;
+      stats[2] = (S > 0) ? a + offset : LLONG_MAX;
     }
-    stats[0] = t;
-    stats[1] = m;
-    stats[2] = (S > 0) ? a + offset : LLONG_MAX;
   }
   __syncthreads();
 }
@@ -84,12 +80,9 @@ __device__ void block_screen_apply(const int64_t* __restrict__ f, int64_t S,
     const unsigned bal = __ballot_sync(0xffffffffu, pass);
     if (lane == 0) s_cnt[warp] = __popc(bal);
     __syncthreads();
-    int before = 0, total = 0;
-    for (int i = 0; i < WARPS; ++i) {
-      int c = s_cnt[i];
-      before += (i < warp) ? c : 0;
-      total += c;
-    }
+    const int c = s_cnt[lane];  // WARPS == 32: one count per lane
+    const int before = __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
+    const int total = __reduce_add_sync(0xffffffffu, c);
     if (pass) idx[base + before + __popc(bal & ((1u << lane) - 1u))] = (int32_t)b;
     base += total;
     __syncthreads();
