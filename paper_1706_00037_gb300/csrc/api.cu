@@ -63,7 +63,8 @@ const int8_t* kernel_readable(const int8_t* p) {
 }
 
 // AUTO: the staged or the fused tensor-core evaluation, whichever is faster
-// for this size (ubqp::eval_auto_fused).
+// for this size (ubqp::eval_auto_fused).  For small instances ubqp_eval then
+// launches eval_small in its place (ubqp::eval_auto_small).
 int resolve_path(const ubqp_q* q, int64_t S, int path) {
   if (path != UBQP_EVAL_AUTO) return path;
   return (q && ubqp::eval_auto_fused(q->n_tc, S)) ? UBQP_EVAL_TC : UBQP_EVAL_TC_STAGED;
@@ -368,6 +369,7 @@ int ubqp_eval(const ubqp_q* q, const uint64_t* X_dev, int64_t S, int64_t* f_dev,
   UBQP_RANGE("ubqp:eval");
   if (!q || !X_dev || !f_dev) return fail(UBQP_ERR_ARG, "NULL argument");
   if (S < 0) return fail(UBQP_ERR_ARG, "S < 0");
+  const bool small = path == UBQP_EVAL_AUTO && q->tc_ok && ubqp::eval_auto_small(q->n, S);
   path = resolve_path(q, S, path);
   if (path != UBQP_EVAL_TC && path != UBQP_EVAL_PLAIN && path != UBQP_EVAL_TC_STAGED &&
       path != UBQP_EVAL_TC_TMEM)
@@ -394,6 +396,10 @@ int ubqp_eval(const ubqp_q* q, const uint64_t* X_dev, int64_t S, int64_t* f_dev,
   if (ws_bytes < need || (need && !ws))
     return fail(UBQP_ERR_NOMEM, "eval workspace %zu < %zu bytes", ws_bytes, need);
   if (((uintptr_t)ws & 15) != 0) return fail(UBQP_ERR_ARG, "workspace not 16-byte aligned");
+  if (small) {  // the same checks and workspace as the path it stands in for
+    UBQP_CUDA(ubqp::launch_eval_small(q, X_dev, S, f_dev, st));
+    return UBQP_OK;
+  }
   cudaError_t e = ubqp::launch_eval_tc(q, X_dev, S, f_dev, ws, ws_bytes, st, nullptr, fused);
   if (e == cudaErrorNotSupported)
     return fail(UBQP_ERR_UNSUPPORTED, "tensor-core evaluation not available for this size");
@@ -489,8 +495,10 @@ static int ascent_impl(const ubqp_q* q, uint64_t* X_dev, int64_t* f_dev, const i
           ? reinterpret_cast<unsigned long long*>(static_cast<char*>(ws) + as - 256)
           : nullptr;
   float* Y = nullptr;
-  if (ws && ws_bytes >= ubqp::ascent_tc_workspace(q, S) &&
-      (int64_t)coeff_bound(q) * q->n_tc < (1 << 24)) {
+  if (ubqp::ascent_own_startup(q->n, S, q->sm_count)) {
+    next = nullptr;  // every start is resident at once: no counter to zero
+  } else if (ws && ws_bytes >= ubqp::ascent_tc_workspace(q, S) &&
+             (int64_t)coeff_bound(q) * q->n_tc < (1 << 24)) {
     // the start-up's unpacking also zeroes the counter
     cudaError_t e = ubqp::launch_ascent_init_tc(q, X_dev, idx_dev, count_dev, S, ws, ws_bytes,
                                                 &Y, st, nullptr, next);

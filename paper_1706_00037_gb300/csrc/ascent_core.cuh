@@ -240,7 +240,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   for (int w = 0; w < W && !y_g; ++w) {
     uint64_t word = x_g[w] & valid_mask(n, w);
     while (word) {
-      constexpr int RF = C == 1 ? 4 : C == 2 ? 2 : 1;  // rows in flight
+      constexpr int RF = C == 1 ? 8 : C == 2 ? 2 : 1;  // rows in flight
       int ks[RF];
       int nk = 0;
 #pragma unroll

@@ -234,6 +234,18 @@ cudaError_t launch_diversify_batch(const BatchDesc* d, int count, int64_t max_wo
                                    cudaStream_t st);
 cudaError_t launch_eval_plain(const ubqp_q* h, const uint64_t* X, int64_t S,
                               int64_t* f, cudaStream_t st);
+// The evaluation UBQP_EVAL_AUTO launches for small instances (n <= 128, the
+// int8 Q in shared memory; k_eval_plain.cu): the same values in one launch.
+// Its work grows with n S, the tensor-core path's hardly does.  A whole round
+// with it against one without, us: n = 33 S = 1000 34.7 / 38.2, S = 8000 49.1 /
+// 52.9; n = 100 S = 1000 38.8 / 40.1, S = 2500 45.4 / 46.4, S = 4000 51.8 / 50.0;
+// n = 128 S = 1500 42.4 / 42.4, S = 2500 47.9 / 47.6; n = 200 (two registers of x)
+// 48.3 / 45.8.  So the line is n <= 128 and n S <= 2^18.
+inline bool eval_auto_small(int n, int64_t S) {
+  return n <= 128 && S <= 8192 && n * S <= (1 << 18);
+}
+cudaError_t launch_eval_small(const ubqp_q* h, const uint64_t* X, int64_t S, int64_t* f,
+                              cudaStream_t st);
 size_t eval_tc_workspace(const ubqp_q* h, int64_t S);
 cudaError_t eval_tc_upload_tables(ubqp_q* h, cudaStream_t st);
 cudaError_t eval_tc_prepare(ubqp_q* h, cudaStream_t st);
@@ -266,6 +278,15 @@ cudaError_t launch_ascent_init_tc(const ubqp_q* h, const uint64_t* X, const int3
                                   float** Y_out, cudaStream_t st,
                                   const void* mapA_in = nullptr,
                                   unsigned long long* zero_next = nullptr);
+// Small instances with no more starts than the one-warp climb holds at once:
+// the climb sums the start-up's rows itself, and neither the unpacking nor the
+// tensor-core product nor the zeroing of the counter is launched.  A round with
+// and without, us: n = 33 S = 1000 28.9 / 34.7, n = 100 32.5 / 38.8, n = 128 35.3 /
+// 40.5; n = 200 47.4 / 48.3 (random starts, S = 200: 57.5 / 55.6), n = 256 56.5 /
+// 56.3, n = 512 85.0 / 72.2: below 200 the launches cost more than the sums.
+inline bool ascent_own_startup(int n, int64_t S, int sm_count) {
+  return n <= 128 && S <= 10ll * sm_count;
+}
 cudaError_t eval_tc_static_scratch(void** out);
 // mapA_in: a TMA descriptor (128 bytes) of the unpacked starts in ws made by
 // eval_tc_map_A, or nullptr to build one per call.
