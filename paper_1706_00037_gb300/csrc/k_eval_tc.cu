@@ -1580,11 +1580,6 @@ cudaError_t launch_startup_multi(const YInst* yi, int count, int64_t max_items, 
   return cudaGetLastError();
 }
 
-size_t eval_tc_chunk_bytes(int n_tc) {
-  return sizeof(int4) * (make_chunks(n_tc, BN, false).size() + make_chunks_y(n_tc).size() +
-                         make_chunks(n_tc, BN_TS, false).size());
-}
-
 // The three chunk tables of one padded size, built once per process and size.
 struct ChunkTables {
   std::vector<int4> all;  // evaluation, full square, 192-column evaluation
@@ -1605,6 +1600,10 @@ static const ChunkTables& chunk_tables(int n_tc) {
   t.all.insert(t.all.end(), full.begin(), full.end());
   t.all.insert(t.all.end(), ts.begin(), ts.end());
   return cache.emplace(n_tc, std::move(t)).first->second;
+}
+
+size_t eval_tc_chunk_bytes(int n_tc) {
+  return sizeof(int4) * chunk_tables(n_tc).all.size();
 }
 
 // Copy the chunk tables to the device (async on `st`; the host tables live in

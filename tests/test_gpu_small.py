@@ -1,7 +1,9 @@
 """Small instances (n <= 128): the shared-memory evaluation that AUTO launches
 and the climb's own start-up, at the edges of their rules; and the block-wide
 sums and maxima of the screen and the best at sizes around a warp and a block,
-with values that need all 64 bits.  Integer results: the tolerance is zero."""
+with values that need all 64 bits; and the preparation of Q from rows at any
+alignment, with the start-up product built on it, at the edges of its tiles.
+Integer results: the tolerance is zero."""
 import numpy as np
 import pytest
 import torch
@@ -80,3 +82,40 @@ def test_block_reductions(S, kind):
     bx, bf = ubqp.best(f, X)
     assert bf.cpu().tolist() == [int(v.max()), int(v.argmax())]
     assert torch.equal(bx, X[int(v.argmax())])
+
+
+@pytest.mark.parametrize("off", [0, 1, 3])
+@pytest.mark.parametrize("n", [1, 2, 3, 63, 64, 65, 68, 127, 130, 197, 257, 322, 515])
+def test_prepare_rows_at_any_alignment(n, off):
+    Q = instance(n, "any")
+    flat = torch.full((n * n + off,), 77, dtype=torch.int8, device="cuda")
+    flat[off:] = torch.from_numpy(Q).cuda().flatten()
+    inst = ubqp.Instance(flat[off:].view(n, n))
+    assert inst.max_abs == int(np.abs(Q.astype(np.int32)).max())
+    S = 150
+    X = ubqp.diversify(inst, S, mode=ubqp.RANDOM, seed=n)
+    j = torch.arange(n, device="cuda")
+    bits = ((X[:, j // 64] >> (j % 64)) & 1).double()
+    y = bits @ torch.from_numpy(Q).cuda().double()
+    want = (y * bits).sum(1).long()
+    for path in (ubqp.EVAL_PLAIN, ubqp.EVAL_TC_STAGED, ubqp.EVAL_TC):  # the int8 copy, Q'
+        assert torch.equal(ubqp.eval(inst, X, path=path), want)
+    # one move from the tensor-core start-up (Q' and its transpose) against one without
+    idx = torch.zeros(1600, dtype=torch.int32, device="cuda")
+    idx[:S] = torch.arange(S, dtype=torch.int32, device="cuda")
+    cnt = torch.full((1,), S, dtype=torch.int64, device="cuda")
+    got = []
+    for use in (True, False):
+        Xa, f = X.clone(), want.clone()
+        ubqp.ascent(inst, Xa, f, idx, cnt, 1, use_ws=use)
+        got.append((Xa, f))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    x0 = ubqp.first_derivative(inst)
+    x0 = ((x0[j // 64] >> (j % 64)) & 1).bool().cpu().numpy()
+    assert np.array_equal(x0, Q.astype(np.int64).sum(1) > 0)
+    if n > 1:  # one element off the symmetric value, anywhere in a tile
+        for r, c in ((0, n - 1), (n - 1, 0), (n // 2, n // 2 - 1)):
+            bad = flat.clone()
+            bad[off + r * n + c] = (int(Q[r, c]) + 129) % 256 - 128
+            with pytest.raises(Exception, match="symmetric"):
+                ubqp.Instance(bad[off:].view(n, n))
