@@ -56,6 +56,11 @@ constexpr int KCH = 16;  // max K steps (of BK) per work unit
 constexpr int THREADS = 192;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
+// Y mode: behind the barriers, 32 x 32 floats per epilogue warp (rows of 36, so
+// that both directions are free of bank conflicts)
+constexpr int YST_LD = 36;
+constexpr int YST_OFF = STAGES * STAGE_BYTES + 256;
+constexpr int SMEM_BYTES_Y = SMEM_BYTES + 4 * 32 * YST_LD * 4;
 // fused variant: two more warps build the A operand from the solution bits,
 // with a 256-entry byte -> 8 bf16 table in shared memory
 constexpr int A_WRITERS = 128;  // one row of the A tile per thread
@@ -304,6 +309,32 @@ __device__ __forceinline__ void expand16(uint32_t x16, uint32_t (&v)[8]) {
   for (int j = 0; j < 8; ++j) v[j] = ((m >> (2 * j)) & 0x10001u) * 0x3F80u;
 }
 
+// Adds a warp's 32 x 32 accumulator block (lane = row, r[c] = column c), halved, to
+// Y: y points at its first element, `left` rows from there exist.  The tensor
+// memory hands each lane a row of its own, and adding from there touched 32 rows
+// per instruction, 16 bytes each; through shared memory (st: the warp's 32 rows of
+// YST_LD floats) eight lanes add 128 consecutive bytes of one row.  Start-up and
+// first move of 500 starts, us: n = 4000 49.8 -> 45.7, n = 7000 109.2 -> 94.8 (1000
+// starts 192.1 -> 159.4); 450 starts at n = 2500 26.2 -> 24.2.
+__device__ __forceinline__ void y_add_block(float* st, const uint32_t (&r)[32], float* y,
+                                            int64_t ldy, int64_t left) {
+  const int lane = threadIdx.x & 31;
+  float4* w = reinterpret_cast<float4*>(st + lane * YST_LD);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    w[i] = make_float4(0.5f * __uint_as_float(r[4 * i]), 0.5f * __uint_as_float(r[4 * i + 1]),
+                       0.5f * __uint_as_float(r[4 * i + 2]), 0.5f * __uint_as_float(r[4 * i + 3]));
+  __syncwarp();
+  const int r0 = lane >> 3, c = 4 * (lane & 7);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int row = 4 * i + r0;
+    const float4 v = *reinterpret_cast<const float4*>(st + row * YST_LD + c);
+    if (row < left) atomicAdd(reinterpret_cast<float4*>(y + row * ldy + c), v);
+  }
+  __syncwarp();
+}
+
 // YMODE = false: f_s += sum_j x_sj D_sj over the lower block triangle (Evaluate).
 // YMODE = true:  Y = (Xe Q'^t + Xe Q') / 2 = Xe Q (Q symmetric), N-block J
 // taking K steps [0, 4(J+1)) of Q' (tmB) and then [4J, n_tc/64) of Q'^t
@@ -542,20 +573,14 @@ eval_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int64_t s = (int64_t)un.mt * BM + row;
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN);
       if (YMODE) {
-        float* yrow = Y + s * ldy + (int64_t)un.nb * BN;
+        const int64_t s0 = (int64_t)un.mt * BM + q * 32;
+        float* y0 = Y + s0 * ldy + (int64_t)un.nb * BN;
+        float* st = reinterpret_cast<float*>(smem + YST_OFF) + q * 32 * YST_LD;
 #pragma unroll 1
         for (int cc = 0; cc < BN / 32; ++cc) {
           uint32_t r[32];
           tmem_ld32(base + (uint32_t)(cc * 32), r);
-          if (s < rows) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              atomicAdd(reinterpret_cast<float4*>(yrow + cc * 32 + 4 * i),
-                        make_float4(0.5f * __uint_as_float(r[4 * i]),
-                                    0.5f * __uint_as_float(r[4 * i + 1]),
-                                    0.5f * __uint_as_float(r[4 * i + 2]),
-                                    0.5f * __uint_as_float(r[4 * i + 3])));
-          }
+          y_add_block(st, r, y0 + cc * 32, ldy, rows - s0);
         }
         tc_fence_before();
         __syncwarp();
@@ -963,7 +988,6 @@ eval_tc_multi_y_kernel(const YInst* __restrict__ yi, const CUtensorMap* __restri
   } else {
     // ---------------- epilogue: warps 2..5 cover TMEM lanes 64-95, 96-127, 0-31, 32-63
     const int q = warp & 3;
-    const int row = q * 32 + lane;
     int t = 0;
     for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
       const MUnit un = units[u];
@@ -977,22 +1001,15 @@ eval_tc_multi_y_kernel(const YInst* __restrict__ yi, const CUtensorMap* __restri
       const bool got = mbar_wait(&tfull[a], aphase, abort_flag, err);
       if (!__all_sync(0xffffffffu, got)) break;
       tc_fence_after();
-      const int64_t s = (int64_t)un.mt * BM + row;
+      const int64_t s0 = (int64_t)un.mt * BM + q * 32;
       const uint32_t base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN);
-      float* yrow = e.Y + s * (int64_t)e.n_tc + (int64_t)un.nb * BN;
+      float* y0 = e.Y + s0 * (int64_t)e.n_tc + (int64_t)un.nb * BN;
+      float* st = reinterpret_cast<float*>(smem + YST_OFF) + q * 32 * YST_LD;
 #pragma unroll 1
       for (int cc = 0; cc < BN / 32; ++cc) {
         uint32_t r[32];
         tmem_ld32(base + (uint32_t)(cc * 32), r);
-        if (s < rows) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            atomicAdd(reinterpret_cast<float4*>(yrow + cc * 32 + 4 * i),
-                      make_float4(0.5f * __uint_as_float(r[4 * i]),
-                                  0.5f * __uint_as_float(r[4 * i + 1]),
-                                  0.5f * __uint_as_float(r[4 * i + 2]),
-                                  0.5f * __uint_as_float(r[4 * i + 3])));
-        }
+        y_add_block(st, r, y0 + cc * 32, e.n_tc, rows - s0);
       }
       tc_fence_before();
       __syncwarp();
@@ -1357,7 +1374,7 @@ cudaError_t set_smem_attr_once() {
   std::call_once(once, [] {
     err = cudaFuncSetAttribute(eval_tc_kernel<YMODE, FUSED>,
                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               FUSED ? SMEM_BYTES_FUSED : SMEM_BYTES);
+                               FUSED ? SMEM_BYTES_FUSED : YMODE ? SMEM_BYTES_Y : SMEM_BYTES);
   });
   return err;
 }
@@ -1562,7 +1579,7 @@ cudaError_t launch_startup_multi(const YInst* yi, int count, int64_t max_items, 
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
     attr = cudaFuncSetAttribute(eval_tc_multi_y_kernel,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES_Y);
   });
   if (attr != cudaSuccess) return attr;
   if (count < 1 || n_units < 1) return cudaSuccess;
@@ -1574,7 +1591,7 @@ cudaError_t launch_startup_multi(const YInst* yi, int count, int64_t max_items, 
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int grid = n_units < sm_count ? n_units : sm_count;
-  eval_tc_multi_y_kernel<<<grid, THREADS, SMEM_BYTES, st>>>(
+  eval_tc_multi_y_kernel<<<grid, THREADS, SMEM_BYTES_Y, st>>>(
       yi, reinterpret_cast<const CUtensorMap*>(mapsA), reinterpret_cast<const CUtensorMap*>(mapsB),
       reinterpret_cast<const CUtensorMap*>(mapsU), units, n_units, err);
   return cudaGetLastError();
@@ -1690,7 +1707,7 @@ cudaError_t launch_ascent_init_tc(const ubqp_q* h, const uint64_t* X, const int3
   const int n_units = h->tc_nchunks_y * m_tiles;
   const int grid = n_units < h->sm_count ? n_units : h->sm_count;
   if ((e = launch_product<true, false>(
-           grid, THREADS, SMEM_BYTES, st, mapA, *reinterpret_cast<const CUtensorMap*>(h->tc_mapB),
+           grid, THREADS, SMEM_BYTES_Y, st, mapA, *reinterpret_cast<const CUtensorMap*>(h->tc_mapB),
            *reinterpret_cast<const CUtensorMap*>(h->tc_mapU), X, h->n, h->W, S, m_tiles,
            reinterpret_cast<const int4*>(h->tc_chunks) + h->tc_nchunks, h->tc_nchunks_y, nullptr,
            count, Y, (int64_t)h->n_tc, h->err)))

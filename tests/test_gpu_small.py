@@ -119,3 +119,22 @@ def test_prepare_rows_at_any_alignment(n, off):
             bad[off + r * n + c] = (int(Q[r, c]) + 129) % 256 - 128
             with pytest.raises(Exception, match="symmetric"):
                 ubqp.Instance(bad[off:].view(n, n))
+
+
+@pytest.mark.parametrize("count", [0, 1, 31, 32, 33, 127, 128, 129, 160])
+def test_startup_product_rows(count):
+    """The rows of Y that the start-up product adds to, at the edges of a warp's
+    32 rows and of a tile's 128: one move from it against one without."""
+    n, S = 515, 200
+    inst = ubqp.Instance(torch.from_numpy(instance(n, "any")).cuda())
+    X = ubqp.diversify(inst, S, mode=ubqp.RANDOM, seed=count)
+    f0 = ubqp.eval(inst, X)
+    idx = torch.randperm(S, device="cuda").int()
+    cnt = torch.full((1,), count, dtype=torch.int64, device="cuda")
+    got = []
+    for use in (True, False):
+        Xa, f = X.clone(), f0.clone()
+        ubqp.ascent(inst, Xa, f, idx, cnt, 1, use_ws=use)
+        got.append((Xa, f))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    assert int((got[0][1] != f0).sum()) <= count
