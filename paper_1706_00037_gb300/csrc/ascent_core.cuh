@@ -63,6 +63,10 @@ __device__ __forceinline__ void runners_up(int2 r, int first, int* cand) {
 // start-up rows and 2^14 relinking steps, so it never reaches a real key.
 constexpr int kKeyBits = 5;
 constexpr int kOutKey = -(1 << 30);
+// Below every real key and above every kOutKey: a thread without candidates
+// enters the reduction with it, and in the block-wide one, 2^2 times as large,
+// it still fits.
+constexpr int kFloorKey = -(1 << 28);
 
 // The flip of the owned element ek, found by a binary decision on its local
 // index (about log2(E) branches instead of E predicated operations): its key
@@ -93,7 +97,9 @@ struct Group<32> {
   __device__ __forceinline__ int rank() const { return threadIdx.x & 31; }
   int2 mine;  // this lane's entry of the last reduction
   // returns {max gain, 2k + x_k} over the group
-  __device__ __forceinline__ int2 reduce(int gain, int jx) {
+  template <int CB>
+  __device__ __forceinline__ int2 reduce(int rank, int jx) {
+    const int gain = rank >> CB;
     const int m = __reduce_max_sync(0xffffffffu, gain);
     const int c = __reduce_min_sync(0xffffffffu, gain == m ? jx : INT_MAX);
     mine = make_int2(gain, jx);
@@ -117,19 +123,30 @@ struct Group {
   int parity;
   __device__ __forceinline__ int rank() const { return threadIdx.x; }
   int2 mine;  // warp `lane`'s winner in the last reduction
-  // returns {max gain, 2k + x_k} over the group
-  __device__ __forceinline__ int2 reduce(int gain, int jx) {
+  // returns {max gain, 2k + x_k} over the group.  rank orders the threads'
+  // entries by gain, then by chunk (2^CB gain + the chunks above the entry's),
+  // and within a chunk a lower lane has the lower index, so one maximum of
+  // {rank, 31 - lane} finds the warp's first winner, which writes its own entry.
+  // (With a second reduction for the index, climbs of n = 1025, 510 starts: 136.2
+  // -> 132.6 us; 2500, 542: 352.2 -> 348.7; 7000, 641: 2617 -> 2573.)
+  template <int CB>
+  __device__ __forceinline__ int2 reduce(int rank, int jx) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int m = __reduce_max_sync(0xffffffffu, gain);
-    const int c = __reduce_min_sync(0xffffffffu, gain == m ? jx : INT_MAX);
-    if (lane == 0) rec[parity][warp] = make_int2(m, c);
+    const int key = (rank << 5) | (31 - lane);
+    // predicated, not a branch: divergence costs more than the store
+    asm volatile(
+        "{\n .reg .pred p;\n setp.eq.s32 p, %0, %1;\n @p st.shared.v2.s32 [%2], {%3, %4};\n}\n" ::"r"(
+            key),
+        "r"(__reduce_max_sync(0xffffffffu, key)),
+        "r"((uint32_t)__cvta_generic_to_shared(&rec[parity][warp])), "r"(rank), "r"(jx)
+        : "memory");
     __syncthreads();
     const int2 r = lane < NW ? rec[parity][lane] : make_int2(INT_MIN, INT_MAX);
     const int m2 = __reduce_max_sync(0xffffffffu, r.x);
     const int c2 = __reduce_min_sync(0xffffffffu, r.x == m2 ? r.y : INT_MAX);
     parity ^= 1;
     mine = r;
-    return make_int2(m2, c2);
+    return make_int2(m2 >> CB, c2);
   }
   // runners-up of the last reduction among the warps' winners
   template <int R>
@@ -273,13 +290,14 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   // ---- first argmax
   int km[NG][2];
 #pragma unroll
-  for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = INT_MIN;
+  for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = kFloorKey;
 #pragma unroll
   for (int e = 0; e < E; e += 2)
     km[e >> 5][(e >> 1) & 1] = __vimax3_s32(km[e >> 5][(e >> 1) & 1], key[e], key[e + 1]);
   // the group's {max gain, 2k + x_k} from each thread's best key: the first
   // key group that attains the thread's largest gain (lower groups hold lower
   // indices)
+  constexpr int CB = C == 1 ? 0 : C == 2 ? 1 : 2;  // bits that count chunks
   auto reduce_key = [&]() {
     int bk = max(km[0][0], km[0][1]), e0 = 31;
     uint32_t xw = xm[0];
@@ -294,7 +312,11 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     }
     const int l = 31 - (bk & 31), e = e0 - (bk & 31);
     const int j = (e >> 4) * CW + 16 * g + (e & 15);
-    return grp.reduce(bk >> kKeyBits, (j << 1) | (int)((xw >> l) & 1u));
+    // (2^CB gain) + (2^CB - 1 - chunk)
+    const int rank = C == 1 ? bk >> kKeyBits
+                     : C == 2 ? bk >> 4
+                              : ((bk >> kKeyBits) << CB) + ((1 << CB) - 1 - (e >> 4));
+    return grp.template reduce<CB>(rank, (j << 1) | (int)((xw >> l) & 1u));
   };
   // Speculation: the next move is often the runner-up of the previous
   // reduction (about 40% of moves at n = 7000), so each move copies this
@@ -415,7 +437,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
                                 (2 * qkk - best.x) * (1 << kKeyBits));
     }
 #pragma unroll
-    for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = INT_MIN;
+    for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = kFloorKey;
 #pragma unroll
     for (int e = 0; e < E; e += 2) {
       key[e] = __dp4a(q[e >> 2], (int)sel[e], key[e]);
