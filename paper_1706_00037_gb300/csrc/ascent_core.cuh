@@ -74,17 +74,22 @@ constexpr int kFloorKey = -(1 << 28);
 // the element's own term of the row update that follows, -2 q_kk, taken off
 // beforehand; its selector changes sign and its x bit flips.  q_kk comes from
 // shared memory, not from the row, so the flip does not wait for the row.
+// The decisions depend on ek alone, which the whole group knows: every lane of
+// the owner's warp takes the same path and only the writes are the owner's
+// (own).  Taken by the owner alone, each level was a divergent branch of its own:
+// climbs of n = 500, 398 starts 79.1 -> 73.5 us; 2500, 3213 starts 1153 -> 1057;
+// 4000, 2193 starts 1824 -> 1679.
 template <int LO, int HI, int E, bool RL>
 __device__ __forceinline__ void flip_tree(int (&key)[E], uint32_t (&sel)[E],
-                                          uint32_t (&xm)[(E + 31) / 32], int ek, int v) {
+                                          uint32_t (&xm)[(E + 31) / 32], int ek, int v, bool own) {
   if constexpr (HI - LO == 1) {
-    key[LO] = RL ? kOutKey : v + (31 - (LO & 31));
-    sel[LO] ^= 0x80u << (8 * (LO & 3));
-    xm[LO >> 5] ^= 1u << (LO & 31);
+    if (own) key[LO] = RL ? kOutKey : v + (31 - (LO & 31));
+    sel[LO] ^= own ? 0x80u << (8 * (LO & 3)) : 0u;
+    xm[LO >> 5] ^= own ? 1u << (LO & 31) : 0u;
   } else {
     constexpr int MID = (LO + HI) / 2;
-    if (ek < MID) flip_tree<LO, MID, E, RL>(key, sel, xm, ek, v);
-    else flip_tree<MID, HI, E, RL>(key, sel, xm, ek, v);
+    if (ek < MID) flip_tree<LO, MID, E, RL>(key, sel, xm, ek, v, own);
+    else flip_tree<MID, HI, E, RL>(key, sel, xm, ek, v, own);
   }
 }
 
@@ -204,6 +209,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   // keys by no more than a real row would.  Row offsets fit 32 bits (n and
   // ldq <= 2^14).
   const uint32_t ld32 = (uint32_t)ldq;
+  const int warp = __shfl_sync(0xffffffffu, g >> 5, 0);  // the same register in every lane
   uint32_t off[C];
 #pragma unroll
   for (int c = 0; c < C; ++c)
@@ -431,10 +437,10 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     }
     // the owner of k flips x_k (when relinking, k leaves the candidates)
     const int kc = k / CW, kr = k - kc * CW;
-    if ((kr >> 4) == g) {
+    if (T == 32 || (kr >> 9) == warp) {
       const int qkk = reinterpret_cast<const int8_t*>(diag)[k];
       flip_tree<0, E, E, RL>(key, sel, xm, kc * 16 + (kr & 15),
-                                (2 * qkk - best.x) * (1 << kKeyBits));
+                             (2 * qkk - best.x) * (1 << kKeyBits), (kr >> 4) == g);
     }
 #pragma unroll
     for (int h = 0; h < NG; ++h) km[h][0] = km[h][1] = kFloorKey;
@@ -821,16 +827,16 @@ struct Climb {
 //        copies, for lists that keep every SM busy: there the issue slots
 //        bound the climb, and the copies cost more than their hits save.
 // Measured on 1000 to 12 000 diversified starts, the passing ones climbed (us,
-// with y, S, C registers -> now): n = 1025, 510 starts 187 -> 136; 2500, 542
-// starts 533 -> 353; 1000, 5638 starts 784 -> 359; 1400, 6069: 1382 -> 677;
-// 2000, 4214: 1406 -> 853; 2500, 3213: 2082 -> 1152; 4000, 2193: 3046 -> 1833;
-// 5000, 4469: 9080 -> 5369; 6000, 2187: 7464 -> 3655; 7000, 54: 1857 -> 1636;
-// 7000, 641: 3364 -> 2606; 7000, 2172: 9610 -> 5243.  The boundary between mid and all lies where
-// a list of that n keeps mid's SMs busy anyway: both take the same time near
-// 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000 starts 2178
-// and 2077), earlier where mid fits only two or three blocks (n = 4800, 600
-// starts: 2387 mid, 2397 all; n = 5800, 300: 2620 and 2682, 600: 3612 and
-// 3000).
+// with y, S, C registers -> now): n = 1025, 510 starts 187 -> 132; 2500, 542
+// starts 533 -> 350; 1000, 5638 starts 784 -> 344; 1400, 6069: 1382 -> 662;
+// 2000, 4214: 1406 -> 836; 2500, 3213: 2082 -> 1055; 4000, 2193: 3046 -> 1675;
+// 5000, 4469: 9080 -> 5260; 6000, 2187: 7464 -> 3584; 7000, 54: 1857 -> 1624;
+// 7000, 641: 3364 -> 2558; 7000, 2172: 9610 -> 5045.  The boundary between mid
+// and all lies where a list of that n keeps mid's SMs busy anyway: both take the
+// same time near 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000
+// starts 2178 and 2077), earlier where mid fits only two or three blocks (n =
+// 4800, 600 starts: 2387 mid, 2397 all; n = 5800, 300: 2620 and 2682, 600: 3612
+// and 3000).
 template <bool TR>
 cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
                                  const int64_t* count, int64_t S, int32_t max_flips,
