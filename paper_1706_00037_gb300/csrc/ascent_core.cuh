@@ -303,7 +303,8 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   // the group's {max gain, 2k + x_k} from each thread's best key: the first
   // key group that attains the thread's largest gain (lower groups hold lower
   // indices)
-  constexpr int CB = C == 1 ? 0 : C == 2 ? 1 : 2;  // bits that count chunks
+  // bits that count chunks (one warp looks for the lowest index itself)
+  constexpr int CB = T == 32 || C == 1 ? 0 : C == 2 ? 1 : C <= 4 ? 2 : 3;
   auto reduce_key = [&]() {
     int bk = max(km[0][0], km[0][1]), e0 = 31;
     uint32_t xw = xm[0];
@@ -318,10 +319,10 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     }
     const int l = 31 - (bk & 31), e = e0 - (bk & 31);
     const int j = (e >> 4) * CW + 16 * g + (e & 15);
-    // (2^CB gain) + (2^CB - 1 - chunk)
-    const int rank = C == 1 ? bk >> kKeyBits
-                     : C == 2 ? bk >> 4
-                              : ((bk >> kKeyBits) << CB) + ((1 << CB) - 1 - (e >> 4));
+    // 2^CB gain + 2^CB - 1 - chunk
+    const int rank = CB == 0   ? bk >> kKeyBits
+                     : CB == 1 ? bk >> 4
+                               : ((bk >> kKeyBits) << CB) + ((1 << CB) - 1 - (e >> 4));
     return grp.template reduce<CB>(rank, (j << 1) | (int)((xw >> l) & 1u));
   };
   // Speculation: the next move is often the runner-up of the previous
@@ -823,14 +824,18 @@ struct Climb {
 //        capacity.
 //   mid  two chunks per thread and several blocks per SM, whose waits cover
 //        one another.
-//   all  the fewest warps that hold n (one up to n = 2048) without runner-up
-//        copies, for lists that keep every SM busy: there the issue slots
-//        bound the climb, and the copies cost more than their hits save.
+//   all  few warps per start, and elements beyond n in as few threads as the
+//        registers allow (one warp up to n = 2560, 80 elements a thread), without
+//        runner-up copies, for lists that keep every SM busy: there the issue
+//        slots bound the climb, and the copies cost more than their hits save.
+//        (n = 2500, 3213 starts: two warps of 48 elements a thread 1059, one of 80
+//        996; n = 5000, 4469 starts: 96 threads of 64 5255, with 1144 elements
+//        beyond n, 160 of 32 4659; n = 1400: seven blocks per SM 662, six 634.)
 // Measured on 1000 to 12 000 diversified starts, the passing ones climbed (us,
 // with y, S, C registers -> now): n = 1025, 510 starts 187 -> 132; 2500, 542
-// starts 533 -> 350; 1000, 5638 starts 784 -> 344; 1400, 6069: 1382 -> 662;
-// 2000, 4214: 1406 -> 836; 2500, 3213: 2082 -> 1055; 4000, 2193: 3046 -> 1675;
-// 5000, 4469: 9080 -> 5260; 6000, 2187: 7464 -> 3584; 7000, 54: 1857 -> 1624;
+// starts 533 -> 350; 1000, 5638 starts 784 -> 344; 1400, 6069: 1382 -> 634;
+// 2000, 4214: 1406 -> 832; 2500, 3213: 2082 -> 996; 4000, 2193: 3046 -> 1675;
+// 5000, 4469: 9080 -> 4659; 6000, 2187: 7464 -> 3584; 7000, 54: 1857 -> 1624;
 // 7000, 641: 3364 -> 2558; 7000, 2172: 9610 -> 5045.  The boundary between mid
 // and all lies where a list of that n keeps mid's SMs busy anyway: both take the
 // same time near 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000
@@ -869,13 +874,13 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
 #define UBQP_C(TT, CC, RR, OCC) Climb<TT, CC, RR, OCC, TR>{}
   if (n <= 512) return two(UBQP_C(32, 1, 1, 8), UBQP_C(32, 1, 0, 10), full);
   if (n <= 1024) return two(UBQP_C(64, 1, 1, 8), UBQP_C(32, 2, 0, 8), full);
-  if (n <= 1536) return tiers(UBQP_C(96, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 3, 0, 7), full);
+  if (n <= 1536) return tiers(UBQP_C(96, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 3, 0, 6), full);
   if (n <= 2048) return tiers(UBQP_C(128, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 4, 0, 5), full);
-  if (n <= 2560) return tiers(UBQP_C(160, 1, 1, 3), UBQP_C(96, 2, 1, 4), UBQP_C(64, 3, 0, 7), full);
+  if (n <= 2560) return tiers(UBQP_C(160, 1, 1, 3), UBQP_C(96, 2, 1, 4), UBQP_C(32, 5, 0, 4), full);
   if (n <= 3072) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(96, 2, 1, 4), UBQP_C(64, 3, 0, 7), full);
   if (n <= 4096) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(128, 2, 1, 4), UBQP_C(64, 4, 0, 5), full);
   if (n <= 5120)
-    return tiers(UBQP_C(160, 2, 1, 1), UBQP_C(160, 2, 1, 3), UBQP_C(96, 4, 0, 3), 4ll * h->sm_count);
+    return tiers(UBQP_C(160, 2, 1, 1), UBQP_C(160, 2, 1, 3), UBQP_C(160, 2, 0, 4), 4ll * h->sm_count);
   if (n <= 6144)
     return tiers(UBQP_C(192, 2, 1, 1), UBQP_C(192, 2, 1, 2), UBQP_C(96, 4, 0, 3), 2ll * h->sm_count);
   if (n <= 7168)

@@ -28,20 +28,23 @@
 // and flips its x bit; it takes q_kk from a copy of the diagonal in shared
 // memory, so that nothing but the update itself waits for the row (with q_kk
 // taken from the row the owner's branches came after the load: n = 7000, 2172
-// starts 6.53 -> 5.24 ms, 54 starts 1.70 -> 1.64).  Rows are read from L2 (the int8 Q of one instance,
-// e.g. 49 MB at n = 7000, stays resident there); nothing per move goes to HBM.
+// starts 6.53 -> 5.24 ms, 54 starts 1.70 -> 1.64).  Rows are read from L2 (the
+// int8 Q of one instance, e.g. 49 MB at n = 7000, stays resident there); nothing
+// per move goes to HBM.
 //
 // What bounds it.  With few starts the chain of moves is latency-bound: per
 // move a dependent L2 row fetch, the update and a block-wide reduction (n =
-// 7000, 54 starts: 763 cycles per move, 1.64 ms; 863 and 1.85 with y, S and C
+// 7000, 54 starts: 757 cycles per move, 1.62 ms; 863 and 1.85 with y, S and C
 // registers).  The loads of the row are issued before anything else of the
 // move, its end test included; the runner-up reduction, the selectors' flip and
-// the owner's branches run in their shadow.  The fetch is taken off the chain when the move was predicted: every move also
-// copies the row of the reduction's runner-up into shared memory, and the next
-// move is that row often enough (about 40% at n = 7000) to pay for the copies.
+// the owner's branches run in their shadow.  The fetch is taken off the chain
+// when the move was predicted: every move also copies the row of the reduction's
+// runner-up into shared memory, and the next move is that row often enough (about
+// 40% at n = 7000) to pay for the copies.
 // With many starts the issue slots and the latency of 12 to 20 warps bound it
-// (n = 1400, 6069 starts: about 185 warp instructions per move, 97 cycles per
-// move and SM, 0.68 ms; 199 cycles and 1.38 ms with y, S and C registers).  launch_ascent_shaped picks the group shape by n and count.
+// (n = 1400, 6069 starts: about 185 warp instructions per move, 91 cycles per
+// move and SM, 0.63 ms; 199 cycles and 1.38 ms with y, S and C registers).
+// launch_ascent_shaped picks the group shape by n and count.
 //
 // Start-up: y = Q x of every listed start comes from the tensor-core product of
 // the ascent workspace when given (exact integers in fp32), else each group
@@ -130,7 +133,7 @@ bool ascent_packed_supported(int T, int C) { return T == 256 && (C == 1 || C == 
 // a kernel per class keeps each class's registers to what its n needs (C = 2:
 // 20 warps per SM, C = 4: 12), and the classes' launches share the chip on
 // streams of their own (32 instances n ~ U[200, 2500], 1024 starts each:
-// 4.38 -> 3.42 ms per run, 6.58 with y, S, C registers).
+// 4.38 -> 3.42 ms per run, 6.58 with y, S, C registers; 2.61 now).
 cudaError_t launch_ascent_batch_packed(const BatchDesc* d, const int2* items, const int4* ranges,
                                        int cls, const int64_t* n_items, int64_t most,
                                        int64_t batch_most, int32_t max_flips, int sm_count,
@@ -149,10 +152,11 @@ cudaError_t launch_ascent_batch_packed(const BatchDesc* d, const int2* items, co
   switch (cls) {
     case 0: return both(UBQP_PK(32, 1, 1, 8), UBQP_PK(32, 1, 0, 10));
     case 1: return both(UBQP_PK(64, 1, 1, 8), UBQP_PK(32, 2, 0, 8));
-    case 2: return both(UBQP_PK(96, 1, 1, 4), UBQP_PK(32, 3, 0, 7));
+    case 2: return both(UBQP_PK(96, 1, 1, 4), UBQP_PK(32, 3, 0, 6));
     case 3: return both(UBQP_PK(128, 1, 1, 4), UBQP_PK(32, 4, 0, 5));
-    case 4: return both(UBQP_PK(96, 2, 1, 4), UBQP_PK(64, 3, 0, 7));
-    case 5: return both(UBQP_PK(128, 2, 1, 4), UBQP_PK(64, 4, 0, 5));
+    case 4: return both(UBQP_PK(96, 2, 1, 4), UBQP_PK(32, 5, 0, 4));
+    case 5: return both(UBQP_PK(96, 2, 1, 4), UBQP_PK(64, 3, 0, 7));
+    case 6: return both(UBQP_PK(128, 2, 1, 4), UBQP_PK(64, 4, 0, 5));
   }
 #undef UBQP_PK
   return cudaErrorInvalidValue;

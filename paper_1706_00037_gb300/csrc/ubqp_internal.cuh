@@ -357,8 +357,8 @@ cudaError_t launch_ascent_batch(const BatchDesc* d, const int2* items, const int
 // n.  Larger instances are left out of the list and climbed one launch per
 // instance (launch_ascent): their own shapes per count are worth more than a
 // shared launch (n = 5000, ~450 passers: 1.40 against 2.01 ms).
-constexpr int kPackedClasses = 6;
-__host__ __device__ constexpr int packed_max_n(int c) { return c < 4 ? 512 * (c + 1) : 1024 * (c - 1); }
+constexpr int kPackedClasses = 7;
+__host__ __device__ constexpr int packed_max_n(int c) { return c < 6 ? 512 * (c + 1) : 4096; }
 __host__ __device__ inline bool packed_own_climb(int n) {
   return n > packed_max_n(kPackedClasses - 1);
 }

@@ -87,7 +87,8 @@ def test_packed_classes_equal_single_solves(S):
     """The packed batch climb at the edges of its size classes, with few starts
     in all and with more than ten per SM."""
     insts = [ubqp.Instance(torch.from_numpy(instance(n, "small")).cuda())
-             for n in (512, 513, 1024, 1025, 1536, 1537, 2048, 2049, 3072, 3073, 4096, 4097)]
+             for n in (512, 513, 1024, 1025, 1536, 1537, 2048, 2049, 2560, 2561, 3072, 3073, 4096,
+                       4097)]
     p = ubqp.make_params(S, 0.25, seed=5)
     batch = ubqp.Batch(insts, p)
     batch.set(256, 2, packed=True)
