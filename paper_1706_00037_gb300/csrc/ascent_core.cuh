@@ -818,30 +818,30 @@ struct Climb {
 // there are.  The count is known only on the device, so for a list that may
 // exceed a shape's range several launches are made, each climbing only for its
 // own range of counts; the others return at once (about 2 us).
-//   few  the shortest chain of moves: enough threads to hold n with 16 (32
-//        above n = 2560) elements each, runner-up rows copied, registers for as
-//        many blocks per SM as that leaves; for lists up to its resident
-//        capacity.
+//   few  the shortest chain of moves: mostly 16 elements per thread, registers for
+//        as many blocks per SM as that leaves; for lists up to its resident
+//        capacity.  (n = 5000, 16 starts: 160 threads of 32 elements 1083, 320 of
+//        16 970; 256 starts 1467 -> 1172.)
 //   mid  two chunks per thread and several blocks per SM, whose waits cover
 //        one another.
+// Neither copies the runner-up's row any more (R = 0): with the cheaper flip and
+// reduction the runner-up's reductions and copies cost every move more than the
+// 40% of moves that hit saved (with and without: n = 1025, 510 starts 131 -> 113; 2500,
+// 542 starts 351 -> 270; 7000, 54 starts 1630 -> 1580, 641 starts 2567 -> 2192).
 //   all  few warps per start, and elements beyond n in as few threads as the
-//        registers allow (one warp up to n = 2560, 80 elements a thread), without
-//        runner-up copies, for lists that keep every SM busy: there the issue
+//        registers allow (one warp up to n = 2560, 80 elements a thread), for lists that keep every SM busy: there the issue
 //        slots bound the climb, and the copies cost more than their hits save.
 //        (n = 2500, 3213 starts: two warps of 48 elements a thread 1059, one of 80
 //        996; n = 5000, 4469 starts: 96 threads of 64 5255, with 1144 elements
 //        beyond n, 160 of 32 4659; n = 1400: seven blocks per SM 662, six 634.)
 // Measured on 1000 to 12 000 diversified starts, the passing ones climbed (us,
-// with y, S, C registers -> now): n = 1025, 510 starts 187 -> 132; 2500, 542
-// starts 533 -> 350; 1000, 5638 starts 784 -> 344; 1400, 6069: 1382 -> 634;
+// with y, S, C registers -> now): n = 1025, 510 starts 187 -> 113; 2500, 542
+// starts 533 -> 270; 1000, 5638 starts 784 -> 344; 1400, 6069: 1382 -> 634;
 // 2000, 4214: 1406 -> 832; 2500, 3213: 2082 -> 996; 4000, 2193: 3046 -> 1675;
-// 5000, 4469: 9080 -> 4659; 6000, 2187: 7464 -> 3584; 7000, 54: 1857 -> 1624;
-// 7000, 641: 3364 -> 2558; 7000, 2172: 9610 -> 5045.  The boundary between mid
-// and all lies where a list of that n keeps mid's SMs busy anyway: both take the
-// same time near 10 starts per SM (n = 2400: 1000 starts 1239 mid, 1322 all; 3000
-// starts 2178 and 2077), earlier where mid fits only two or three blocks (n =
-// 4800, 600 starts: 2387 mid, 2397 all; n = 5800, 300: 2620 and 2682, 600: 3612
-// and 3000).
+// 5000, 4469: 9080 -> 4659; 6000, 2187: 7464 -> 3584; 7000, 54: 1857 -> 1580;
+// 7000, 641: 3364 -> 2192; 7000, 2172: 9610 -> 5045.  The boundary between mid
+// and all lies near 10 starts per SM, where a list of that n keeps mid's SMs busy
+// anyway, and at 2 per SM for 4096 < n <= 6144, where mid fits few blocks.
 template <bool TR>
 cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const int32_t* idx,
                                  const int64_t* count, int64_t S, int32_t max_flips,
@@ -855,9 +855,8 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
   }
   const AscArgs a{h, X, f, idx, count, S, max_flips, flips, Y, next, trace, ldt, st};
   // few: the shortest chain of moves, for lists up to its resident capacity;
-  // mid: several blocks per SM, whose waits cover one another; all: no
-  // runner-up copies and the fewest warps per start, for lists that keep the
-  // whole chip busy (more than `full` starts)
+  // mid: several blocks per SM, whose waits cover one another; all: few warps
+  // per start, for lists that keep the whole chip busy (more than `full` starts)
   auto tiers = [&](auto few, auto mid, auto all, int64_t full) {
     const int64_t cap = std::min(few.capacity(h), full);
     cudaError_t e = few.launch(a, 0, cap);
@@ -872,21 +871,20 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
   };
   const int64_t full = 10ll * h->sm_count;
 #define UBQP_C(TT, CC, RR, OCC) Climb<TT, CC, RR, OCC, TR>{}
-  if (n <= 512) return two(UBQP_C(32, 1, 1, 8), UBQP_C(32, 1, 0, 10), full);
-  if (n <= 1024) return two(UBQP_C(64, 1, 1, 8), UBQP_C(32, 2, 0, 8), full);
-  if (n <= 1536) return tiers(UBQP_C(96, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 3, 0, 6), full);
-  if (n <= 2048) return tiers(UBQP_C(128, 1, 1, 4), UBQP_C(64, 2, 1, 8), UBQP_C(32, 4, 0, 5), full);
-  if (n <= 2560) return tiers(UBQP_C(160, 1, 1, 3), UBQP_C(96, 2, 1, 4), UBQP_C(32, 5, 0, 4), full);
-  if (n <= 3072) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(96, 2, 1, 4), UBQP_C(64, 3, 0, 7), full);
-  if (n <= 4096) return tiers(UBQP_C(128, 2, 1, 2), UBQP_C(128, 2, 1, 4), UBQP_C(64, 4, 0, 5), full);
-  if (n <= 5120)
-    return tiers(UBQP_C(160, 2, 1, 1), UBQP_C(160, 2, 1, 3), UBQP_C(160, 2, 0, 4), 4ll * h->sm_count);
+  if (n <= 512) return two(UBQP_C(32, 1, 0, 8), UBQP_C(32, 1, 0, 10), full);
+  if (n <= 1024) return two(UBQP_C(64, 1, 0, 8), UBQP_C(32, 2, 0, 8), full);
+  if (n <= 1536) return tiers(UBQP_C(96, 1, 0, 7), UBQP_C(64, 2, 0, 8), UBQP_C(32, 3, 0, 6), full);
+  if (n <= 2048) return tiers(UBQP_C(128, 1, 0, 4), UBQP_C(64, 2, 0, 8), UBQP_C(32, 4, 0, 5), full);
+  if (n <= 2560) return tiers(UBQP_C(160, 1, 0, 4), UBQP_C(96, 2, 0, 4), UBQP_C(32, 5, 0, 4), full);
+  if (n <= 3072) return tiers(UBQP_C(192, 1, 0, 2), UBQP_C(96, 2, 0, 4), UBQP_C(64, 3, 0, 7), full);
+  if (n <= 4096) return tiers(UBQP_C(256, 1, 0, 2), UBQP_C(128, 2, 0, 4), UBQP_C(64, 4, 0, 5), full);
+  if (n <= 5120) return two(UBQP_C(320, 1, 0, 2), UBQP_C(160, 2, 0, 4), 2ll * h->sm_count);
   if (n <= 6144)
-    return tiers(UBQP_C(192, 2, 1, 1), UBQP_C(192, 2, 1, 2), UBQP_C(96, 4, 0, 3), 2ll * h->sm_count);
+    return tiers(UBQP_C(384, 1, 0, 1), UBQP_C(192, 2, 0, 3), UBQP_C(96, 4, 0, 3), 2ll * h->sm_count);
   if (n <= 7168)
-    return tiers(UBQP_C(224, 2, 1, 1), UBQP_C(256, 2, 1, 2), UBQP_C(128, 4, 0, 3), full);
+    return tiers(UBQP_C(224, 2, 0, 1), UBQP_C(224, 2, 0, 2), UBQP_C(128, 4, 0, 3), full);
   if (n <= 8192)
-    return tiers(UBQP_C(256, 2, 1, 1), UBQP_C(256, 2, 1, 2), UBQP_C(128, 4, 0, 3), full);
+    return tiers(UBQP_C(256, 2, 0, 1), UBQP_C(256, 2, 0, 2), UBQP_C(128, 4, 0, 3), full);
   return UBQP_C(512, 2, 1, 1).launch(a, 0, INT64_MAX);
 #undef UBQP_C
 }

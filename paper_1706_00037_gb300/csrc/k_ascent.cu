@@ -34,11 +34,11 @@
 //
 // What bounds it.  With few starts the chain of moves is latency-bound: per
 // move a dependent L2 row fetch, the update and a block-wide reduction (n =
-// 7000, 54 starts: 757 cycles per move, 1.62 ms; 863 and 1.85 with y, S and C
+// 7000, 54 starts: 737 cycles per move, 1.58 ms; 863 and 1.85 with y, S and C
 // registers).  The loads of the row are issued before anything else of the
 // move, its end test included; the runner-up reduction, the selectors' flip and
 // the owner's branches run in their shadow.  The fetch is taken off the chain
-// when the move was predicted: every move also copies the row of the reduction's
+// when the move was predicted (relinking, and climbs above n = 8192): every move also copies the row of the reduction's
 // runner-up into shared memory, and the next move is that row often enough (about
 // 40% at n = 7000) to pay for the copies.
 // With many starts the issue slots and the latency of 12 to 20 warps bound it
@@ -127,7 +127,7 @@ bool ascent_packed_supported(int T, int C) { return T == 256 && (C == 1 || C == 
 
 // One size class of a packed batch, in the group shapes launch_ascent_shaped
 // uses for lists of that length: with at most 10 starts per SM in the whole
-// batch the ones with runner-up copies, else the fewest warps that hold n.
+// batch the ones with the shorter chains, else the fewest warps that hold n.
 // Packed climbs ran before as one launch of 256-thread blocks split into
 // sub-groups on named barriers, the classes one after another in each block;
 // a kernel per class keeps each class's registers to what its n needs (C = 2:
@@ -150,13 +150,13 @@ cudaError_t launch_ascent_batch_packed(const BatchDesc* d, const int2* items, co
                                          most, lo, hi, sm_count, st);                         \
   }
   switch (cls) {
-    case 0: return both(UBQP_PK(32, 1, 1, 8), UBQP_PK(32, 1, 0, 10));
-    case 1: return both(UBQP_PK(64, 1, 1, 8), UBQP_PK(32, 2, 0, 8));
-    case 2: return both(UBQP_PK(96, 1, 1, 4), UBQP_PK(32, 3, 0, 6));
-    case 3: return both(UBQP_PK(128, 1, 1, 4), UBQP_PK(32, 4, 0, 5));
-    case 4: return both(UBQP_PK(96, 2, 1, 4), UBQP_PK(32, 5, 0, 4));
-    case 5: return both(UBQP_PK(96, 2, 1, 4), UBQP_PK(64, 3, 0, 7));
-    case 6: return both(UBQP_PK(128, 2, 1, 4), UBQP_PK(64, 4, 0, 5));
+    case 0: return both(UBQP_PK(32, 1, 0, 8), UBQP_PK(32, 1, 0, 10));
+    case 1: return both(UBQP_PK(64, 1, 0, 8), UBQP_PK(32, 2, 0, 8));
+    case 2: return both(UBQP_PK(96, 1, 0, 7), UBQP_PK(32, 3, 0, 6));
+    case 3: return both(UBQP_PK(128, 1, 0, 4), UBQP_PK(32, 4, 0, 5));
+    case 4: return both(UBQP_PK(96, 2, 0, 4), UBQP_PK(32, 5, 0, 4));
+    case 5: return both(UBQP_PK(96, 2, 0, 4), UBQP_PK(64, 3, 0, 7));
+    case 6: return both(UBQP_PK(128, 2, 0, 4), UBQP_PK(64, 4, 0, 5));
   }
 #undef UBQP_PK
   return cudaErrorInvalidValue;
