@@ -36,11 +36,12 @@
 // move a dependent L2 row fetch, the update and a block-wide reduction (n =
 // 7000, 54 starts: 737 cycles per move, 1.58 ms; 863 and 1.85 with y, S and C
 // registers).  The loads of the row are issued before anything else of the
-// move, its end test included; the runner-up reduction, the selectors' flip and
-// the owner's branches run in their shadow.  The fetch is taken off the chain
-// when the move was predicted (relinking, and climbs above n = 8192): every move also copies the row of the reduction's
-// runner-up into shared memory, and the next move is that row often enough (about
-// 40% at n = 7000) to pay for the copies.
+// move, its end test included; the selectors' flip and the owner's branches run
+// in their shadow.  Relinking, and climbs above n = 8192, take the fetch off the
+// chain where the move was predicted: every move also copies the row of the
+// reduction's runner-up into shared memory, and the next move is that row about
+// 40% of the time at n = 7000.  The other climbs make no such copies: they cost
+// more per move than the hits save.
 // With many starts the issue slots and the latency of 12 to 20 warps bound it
 // (n = 1400, 6069 starts: about 185 warp instructions per move, 91 cycles per
 // move and SM, 0.63 ms; 199 cycles and 1.38 ms with y, S and C registers).
