@@ -498,8 +498,10 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
 // the registers are sized for.  The kernel climbs only when the number of
 // listed starts lies in [cnt_lo, cnt_hi] and returns at once otherwise, so
 // that two launches of different OCC can share one list, each taking the
-// counts it is faster for, with no host round trip for the count.  A
-// programmatic dependent of the kernel before it on the stream (pdl_wait).
+// counts it is faster for, with no host round trip for the count.  Y has S
+// rows; the starts of a longer list (which has entries outside [0, S)) sum
+// their own start-up.  A programmatic dependent of the kernel before it on the
+// stream (pdl_wait).
 template <int T, int C, int R, bool TR, int OCC>
 __global__ void __launch_bounds__(T, OCC)
 ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
@@ -535,7 +537,7 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
     }
     ascend_one<T, C, R, false, TR>(Q8, ldq, ldy, n, W, X + (int64_t)s * W, f + s, max_flips,
                                    flips ? flips + s : nullptr, err, spec_slots, diag,
-                                   Y ? Y + t * ldy : nullptr, grp, nullptr,
+                                   Y && cnt <= S ? Y + t * ldy : nullptr, grp, nullptr,
                                    TR ? trace + (int64_t)s * ldt : nullptr, ldt);
   }
 }
@@ -582,7 +584,9 @@ ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ it
 
 // Independent warps, one start each (kWarps per block); counts, starts and
 // launch as in the block kernel, the first wave one warp per block over the
-// whole grid before any block's second warp.
+// whole grid before any block's second warp.  (The test for Y's S rows is per
+// entry and in 32 bits here: as in the block kernel it cost the 80-element warps
+// four spilled registers and 2%.)
 template <int C, int R, bool TR, int OCC>
 __global__ void __launch_bounds__(32 * kWarps, OCC)
 ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
@@ -617,7 +621,8 @@ ascent_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                                     flips ? flips + s : nullptr, err,
                                     spec_slots + warp * spec_slot_count<32, C, R>(),
                                     diag + warp * (32 * C),
-                                    Y ? Y + t * ldy : nullptr, grp, nullptr,
+                                    Y && (t >> 31) == 0 && (int)t < (int)S ? Y + t * ldy : nullptr, grp,
+                                    nullptr,
                                     TR ? trace + (int64_t)s * ldt : nullptr, ldt);
   }
 }
@@ -857,15 +862,18 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
   // few: the shortest chain of moves, for lists up to its resident capacity;
   // mid: several blocks per SM, whose waits cover one another; all: few warps
   // per start, for lists that keep the whole chip busy (more than `full` starts)
+  // The last launch made also takes every larger count: a list may be longer
+  // than S when entries in it lie outside [0, S), which the climb reports.
   auto tiers = [&](auto few, auto mid, auto all, int64_t full) {
     const int64_t cap = std::min(few.capacity(h), full);
-    cudaError_t e = few.launch(a, 0, cap);
-    if (e == cudaSuccess && cap < full && S > cap) e = mid.launch(a, cap + 1, full);
+    cudaError_t e = few.launch(a, 0, S > cap ? cap : INT64_MAX);
+    if (e == cudaSuccess && cap < full && S > cap)
+      e = mid.launch(a, cap + 1, S > full ? full : INT64_MAX);
     if (e == cudaSuccess && S > full) e = all.launch(a, full + 1, INT64_MAX);
     return e;
   };
   auto two = [&](auto few, auto all, int64_t full) {
-    cudaError_t e = few.launch(a, 0, full);
+    cudaError_t e = few.launch(a, 0, S > full ? full : INT64_MAX);
     if (e == cudaSuccess && S > full) e = all.launch(a, full + 1, INT64_MAX);
     return e;
   };
