@@ -79,7 +79,6 @@ struct ubqp_batch {
   std::vector<int> alt_nchunks[2];
   // configuration (autotuned)
   int asc_T = 256, asc_C = 1, eval_path = UBQP_EVAL_TC, nstreams = 8;
-  int asc_grid = 0;
   bool packed = false;                   // packed ascent (sub-groups by n)
   int eval_kch = 16;                     // K steps per evaluation work chunk
   // the merged evaluation: start generation and the tensor-core evaluation of
@@ -99,6 +98,7 @@ struct ubqp_batch {
   int n_yunits = 0;
   int64_t max_items = 0;
   int max_n = 0;
+  int64_t min_ldq = UBQP_MAX_N;          // the shortest int8 row of the instances
   std::vector<cudaStream_t> streams;
   std::vector<cudaEvent_t> ev_join;
   cudaEvent_t ev_fork = nullptr;
@@ -225,7 +225,8 @@ int run_body(ubqp_batch* b, cudaStream_t st) {
                                         b->d_nitems, st));
     // the item counter: the second word of the 16-byte item-count slot
     UBQP_BCUDA(ubqp::launch_ascent_batch(b->d_desc, b->d_items, b->d_nitems, b->asc_T, b->asc_C,
-                                         p.max_flips, b->asc_grid,
+                                         4 * b->min_ldq >= 3 * 16ll * b->asc_T * b->asc_C,
+                                         b->count * p.num_starts, p.max_flips, b->sm_count,
                                          reinterpret_cast<unsigned long long*>(b->d_nitems + 1),
                                          st));
   }
@@ -248,7 +249,6 @@ int set_shape(ubqp_batch* b, int T, int C, bool packed = false) {
   b->asc_T = T;
   b->asc_C = C;
   b->packed = packed;
-  b->asc_grid = packed ? 0 : ubqp::ascent_batch_grid(T, C, b->sm_count);
   return UBQP_OK;
 }
 
@@ -293,6 +293,7 @@ int ubqp_batch_create(const ubqp_q* const* qs, int32_t count, const ubqp_params*
       return bfail(UBQP_ERR_ARG, "instances live on different devices");
     }
     b->max_n = std::max(b->max_n, qs[i]->n);
+    b->min_ldq = std::min(b->min_ldq, qs[i]->ldq);
   }
   b->sm_count = qs[0]->sm_count;
   b->order.resize(count);

@@ -544,17 +544,19 @@ ascent_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
 
 // All passing starts of a batch of instances in one persistent launch: item
 // t = (instance, position in its passing list); every instance has n <= 16 T C.
-template <int T, int C, int R>
-__global__ void __launch_bounds__(T, 1)
+// Climbs only when the number of items lies in [lo, hi].
+template <int T, int C, int R, int OCC>
+__global__ void __launch_bounds__(T, OCC)
 ascent_batch_kernel(const BatchDesc* __restrict__ d, const int2* __restrict__ items,
                     const int64_t* __restrict__ n_items, int32_t max_flips,
-                    unsigned long long* __restrict__ next) {
+                    unsigned long long* __restrict__ next, int64_t lo, int64_t hi) {
   __shared__ int2 rec[2][T / 32];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
   __shared__ uint4 diag[T * C];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
   const int64_t cnt = *n_items;
+  if (cnt < lo || cnt > hi) return;  // the other launch's counts
   // the first wave one item per block, the rest from the counter (as in
   // ascent_block_kernel)
   auto take = [&](int64_t t) -> int64_t {
@@ -909,15 +911,14 @@ cudaError_t launch_class(const BatchDesc* d, const int2* items, const int4* rang
   return cudaGetLastError();
 }
 
-template <int T, int C>
-cudaError_t launch_ascent_batch_tc(const BatchDesc* d, const int2* items, const int64_t* n_items,
-                                   int32_t max_flips, int grid, unsigned long long* next,
-                                   cudaStream_t st) {
-  if (next) {
-    cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
-  }
-  ascent_batch_kernel<T, C, kSpecRows><<<grid, T, 0, st>>>(d, items, n_items, max_flips, next);
+template <int T, int C, int R, int OCC>
+cudaError_t launch_batch_shape(const BatchDesc* d, const int2* items, const int64_t* n_items,
+                               int32_t max_flips, unsigned long long* next, int64_t most,
+                               int64_t lo, int64_t hi, int sm_count, cudaStream_t st) {
+  const int64_t grid = std::min<int64_t>(
+      resident_grid(ascent_batch_kernel<T, C, R, OCC>, T, sm_count), most);
+  ascent_batch_kernel<T, C, R, OCC>
+      <<<(unsigned)grid, T, 0, st>>>(d, items, n_items, max_flips, next, lo, hi);
   return cudaGetLastError();
 }
 

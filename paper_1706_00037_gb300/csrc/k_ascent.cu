@@ -95,32 +95,43 @@ bool ascent_batch_supported(int T, int C) {
   return (T == 64 || T == 128 || T == 256 || T == 512) && (C == 1 || C == 2);
 }
 
-int ascent_batch_grid(int T, int C, int sm_count) {
-  int per_sm = 0;
-  cudaError_t e = cudaErrorInvalidValue;
-#define UBQP_OCC(TT, CC)                                                                     \
-  if (T == TT && C == CC)                                                                    \
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                       \
-        &per_sm, ascent_batch_kernel<TT, CC, kSpecRows>, TT, 0);
-  UBQP_OCC(64, 1) UBQP_OCC(64, 2) UBQP_OCC(128, 1) UBQP_OCC(128, 2)
-  UBQP_OCC(256, 1) UBQP_OCC(256, 2) UBQP_OCC(512, 1) UBQP_OCC(512, 2)
-#undef UBQP_OCC
-  if (e != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    per_sm = 1;
-  }
-  return per_sm * sm_count;
-}
-
+// The unpacked climb of a batch: one shape for every instance.  Without
+// runner-up copies: with them, the threads of a group that is wider than an
+// instance's rows copied the same 16 bytes, one request to one L2 slice each (30
+// instances n = 64 to 400, 1024 starts, 256 x 1: 14.5 ms per run, 0.67 without
+// copies), and a full chip gains from dropping them in any case (the same in 64
+// x 1, 0.49 -> 0.25; 8 of n = 3000 in 256 x 1, 4.51 -> 3.36).  Where the rows fill
+// three quarters of a group of 128 threads or more (filled) and there is no more
+// than one start per SM, the copies still hide part of the row fetch (8 of n =
+// 3000, 100 random starts each, about 50 climbed: 757 us with copies, 824 without;
+// 2 of n = 8000: 2370, 2515; but one of n = 9000 in 512 x 2, 0.56 filled: 3049,
+// 2827): those counts keep a launch with copies.
 cudaError_t launch_ascent_batch(const BatchDesc* d, const int2* items, const int64_t* n_items,
-                                int T, int C, int32_t max_flips, int grid,
-                                unsigned long long* next, cudaStream_t st) {
-#define UBQP_ASC(TT, CC)                                                                      \
-  if (T == TT && C == CC)                                                                     \
-    return launch_ascent_batch_tc<TT, CC>(d, items, n_items, max_flips, grid, next, st);
-  UBQP_ASC(64, 1) UBQP_ASC(64, 2) UBQP_ASC(128, 1) UBQP_ASC(128, 2)
-  UBQP_ASC(256, 1) UBQP_ASC(256, 2) UBQP_ASC(512, 1) UBQP_ASC(512, 2)
-#undef UBQP_ASC
+                                int T, int C, bool filled, int64_t most, int32_t max_flips,
+                                int sm_count, unsigned long long* next, cudaStream_t st) {
+  if (next) {
+    cudaError_t e = cudaMemsetAsync(next, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+  }
+  auto pair = [&](auto few, auto many) {
+    cudaError_t e = filled ? few(0, sm_count) : cudaSuccess;
+    if (e == cudaSuccess && (!filled || most > sm_count))
+      e = many(filled ? sm_count + 1 : 0, INT64_MAX);
+    return e;
+  };
+#define UBQP_BT(TT, CC, RR, OCC)                                                                \
+  [&](int64_t lo, int64_t hi) {                                                                 \
+    return launch_batch_shape<TT, CC, RR, OCC>(d, items, n_items, max_flips, next, most, lo,    \
+                                               hi, sm_count, st);                               \
+  }
+#define UBQP_PAIR(TT, CC, OCC) \
+  if (T == TT && C == CC) return pair(UBQP_BT(TT, CC, 1, 1), UBQP_BT(TT, CC, 0, OCC));
+  if (T == 64 && C == 1) return UBQP_BT(64, 1, 0, 10)(0, INT64_MAX);
+  if (T == 64 && C == 2) return UBQP_BT(64, 2, 0, 8)(0, INT64_MAX);
+  UBQP_PAIR(128, 1, 5) UBQP_PAIR(128, 2, 4) UBQP_PAIR(256, 1, 3) UBQP_PAIR(256, 2, 2)
+  UBQP_PAIR(512, 1, 1) UBQP_PAIR(512, 2, 1)
+#undef UBQP_PAIR
+#undef UBQP_BT
   return cudaErrorInvalidValue;
 }
 

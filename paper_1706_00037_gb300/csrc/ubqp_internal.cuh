@@ -347,10 +347,12 @@ cudaError_t launch_screen(const int64_t* f, int64_t S, double lambda, int32_t* i
 cudaError_t launch_screen_batch(const BatchDesc* d, int count, double lambda, cudaStream_t st);
 cudaError_t launch_batch_items(const BatchDesc* d, const int32_t* order, int count, int2* items,
                                int64_t* n_items, cudaStream_t st);
-// next: as in launch_ascent (zeroed here; NULL: round robin)
+// next: as in launch_ascent (zeroed here; NULL: round robin).  filled: every
+// instance's row (ldq) fills three quarters of a group, 16 T C elements.  most:
+// the most items the list can have.
 cudaError_t launch_ascent_batch(const BatchDesc* d, const int2* items, const int64_t* n_items,
-                                int T, int C, int32_t max_flips, int grid,
-                                unsigned long long* next, cudaStream_t st);
+                                int T, int C, bool filled, int64_t most, int32_t max_flips,
+                                int sm_count, unsigned long long* next, cudaStream_t st);
 // Packed batch ascent: the instances fall into classes by n, class c holding
 // packed_max_n(c - 1) < n <= packed_max_n(c), and each class is climbed by a
 // launch of its own (launch_ascent_batch_packed), whose group shape fits its
@@ -380,7 +382,6 @@ cudaError_t launch_ascent_batch_packed(const BatchDesc* d, const int2* items, co
                                        int64_t batch_most, int32_t max_flips, int sm_count,
                                        unsigned long long* next, cudaStream_t st);
 bool ascent_packed_supported(int T, int C);
-int ascent_batch_grid(int T, int C, int sm_count);
 bool ascent_batch_supported(int T, int C);
 cudaError_t launch_best_batch(const BatchDesc* d, int count, cudaStream_t st);
 cudaError_t launch_set_u64(uint64_t* dst, uint64_t v, cudaStream_t st);
