@@ -263,7 +263,10 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
   for (int w = 0; w < W && !y_g; ++w) {
     uint64_t word = x_g[w] & valid_mask(n, w);
     while (word) {
-      constexpr int RF = C == 1 ? 8 : C == 2 ? 2 : 1;  // rows in flight
+      // rows in flight.  Relinking takes as many of the two-chunk rows, its shapes
+      // having the registers (128 x 2, n = 2800: one pair 865 us with 2 rows, 524
+      // with 8; 16 pairs 631, 447; the ascent's have not)
+      constexpr int RF = C == 1 || (RL && C == 2) ? 8 : C == 2 ? 2 : 1;
       int ks[RF];
       int nk = 0;
 #pragma unroll
