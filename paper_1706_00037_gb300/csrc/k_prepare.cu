@@ -15,7 +15,7 @@ namespace ubqp {
 namespace {
 
 constexpr int PT = 64;        // tile edge
-static_assert(UBQP_TC_ALIGN % (2 * PT) == 0, "an even number of tiles");
+static_assert(UBQP_TC_ALIGN % (4 * PT) == 0, "a multiple of four tiles");
 constexpr int PTHREADS = 256;  // 4 threads per tile row, 16 columns each
 
 // Four bytes of row j from column k (zero at or beyond n): one 32-bit load when
@@ -142,8 +142,14 @@ __device__ __forceinline__ void emit_tile(const int8_t (*tile)[PT + 4], int rb, 
 // checks on them inside Q (aligned words and a funnel shift where rows are not).
 // What is left is the latency of a load phase and a store phase per block, five
 // blocks to an SM (eight, with 32 registers, measured slower).
-// The grid folds the triangle of pairs into a rectangle (tiles + 1, tiles / 2);
-// the number of tiles is even.
+// The blocks walk the triangle of pairs along its diagonals, 2 x 2 tiles (a
+// super-tile pair (a, b), b = a + d mod sn for d = 0 .. sn / 2) at a time: blockIdx.y
+// = d sn + a, the last diagonal, d = sn / 2, only half as long.  Along a row, as
+// they ran before, a block's second tile lay 64 rows below the previous block's, so
+// that hundreds of blocks at once touched addresses a multiple of 64 n apart: at n =
+// 16384 and just below (strides of a power of two) 494 and 565 us against 444 and
+// 446 for the unpacked kernel before, 370 now; n = 12288 197 -> 180, n = 6001 and
+// 7000 the same.  The number of tiles is a multiple of four, so sn is even.
 template <bool W4>
 __global__ void __launch_bounds__(PTHREADS)
 prepare_pairs(const int8_t* __restrict__ Q, int n, int64_t ldq_in, int8_t* __restrict__ Q8,
@@ -151,11 +157,9 @@ prepare_pairs(const int8_t* __restrict__ Q, int n, int64_t ldq_in, int8_t* __res
               int32_t* __restrict__ rowsum, unsigned* __restrict__ flags) {
   pdl_enter();
   const int tiles = n_tc / PT;
-  int bi = blockIdx.y, bj = (int)blockIdx.x - 1;
-  if (bj < bi) {
-    bi = tiles - 1 - bi;
-    bj = tiles - 1 - (int)blockIdx.x;
-  }
+  const int sn = tiles / 2, a = (int)blockIdx.y % sn, b = (a + (int)blockIdx.y / sn) % sn;
+  const int bi = 2 * min(a, b) + (int)blockIdx.x / 2, bj = 2 * max(a, b) + (int)blockIdx.x % 2;
+  if (bi > bj) return;
   __shared__ __align__(16) int8_t tile[2][PT][PT + 4];  // T, then U
   const int t = threadIdx.x;
   const int nt = bi == bj ? 1 : 2;
@@ -267,7 +271,8 @@ cudaError_t launch_prepare(const int8_t* Q, int n, int64_t ldq_in, ubqp_q* h,
                   PTHREADS, 0, st>>>(h->rowsum, h->err, h->Q8, h->ldq, n, h->n_tc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const dim3 grid(tiles + 1, tiles / 2);
+  const int sn = tiles / 2;
+  const dim3 grid(4, sn * (sn + 1) / 2);
   if (((uintptr_t)Q & 3) == 0 && (ldq_in & 3) == 0)
     e = launch_pdl(prepare_pairs<true>, grid, dim3(PTHREADS), 0, st, Q, n, ldq_in, h->Q8, h->ldq,
                    h->Qt, h->Qu, h->n_tc, h->rowsum, h->scratch_flags);
