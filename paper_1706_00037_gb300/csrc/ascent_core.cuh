@@ -58,9 +58,14 @@ __device__ __forceinline__ void runners_up(int2 r, int first, int* cand) {
 
 // Keys.  Element e of a thread keeps key = 32 gain + (31 - e % 32), so that an
 // integer maximum over up to 32 keys orders by gain, then by lower index
-// (|gain| < 2^23, so |key| < 2^28).  An element that is no candidate has
-// kOutKey; row updates move it by at most 2^13 per move, over at most 2^14
-// start-up rows and 2^14 relinking steps, so it never reaches a real key.
+// (|gain| < 2^23, so |key| < 2^28).  An element that is no candidate (beyond n,
+// or in relinking one that has been flipped or need not be) has kOutKey, and row
+// updates move that too, since every element of a thread takes them.  Over any
+// number of moves they add up to little: the element's own bit does not change
+// and its selector changes sign only with d, so the sum is +-64 times the change
+// of y = Q x in the column that it reads (column off + e of every row, for chunks
+// beyond the row the same first ones throughout), and y stays within 2^21, so
+// the key within 2^28 of kOutKey: it never reaches a real key.
 constexpr int kKeyBits = 5;
 constexpr int kOutKey = -(1 << 30);
 // Below every real key and above every kOutKey: a thread without candidates
@@ -187,7 +192,7 @@ struct RelinkArgs {
 // the same move machinery, but only variables where x and g differ are
 // candidates, every step is taken whatever its gain, a flipped variable leaves
 // the candidate set, and the best solution strictly between the endpoints is
-// the result.
+// the result.  diag: T C slots of shared memory for the diagonal (RL: unused).
 template <int T, int C, int R, bool RL = false, bool TR = false, class G = Group<T>>
 __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_t ldq,
                                            int64_t ldy, int n,
@@ -258,7 +263,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       sel[e] = (xb ? 0xC0u : 0x40u) << (8 * (o & 3));
       dg[o >> 2] |= (uint32_t)(uint8_t)qjj << (8 * (o & 3));
     }
-    diag[c * T + g] = make_uint4(dg[0], dg[1], dg[2], dg[3]);  // read by this thread only
+    if constexpr (!RL) diag[c * T + g] = make_uint4(dg[0], dg[1], dg[2], dg[3]);
   }
   for (int w = 0; w < W && !y_g; ++w) {
     uint64_t word = x_g[w] & valid_mask(n, w);
@@ -346,6 +351,10 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
       R > 0 ? (uint32_t)__cvta_generic_to_shared(spec_slots) + (uint32_t)g * 16 : 0u;
   int buf = 0;
   int2 best = reduce_key();
+  // every lane of the owner's warp reads q_kk from diag: a block's reduction orders
+  // the writes before it, a warp's holds no barrier.  (Placed here it costs nothing;
+  // right behind the writes, or with the read left to the owner, 1 to 6%.)
+  if constexpr (!RL && T == 32) grp.sync();
 
   int64_t fval = *f_s;
   int flips = 0;
@@ -442,7 +451,7 @@ __device__ __forceinline__ void ascend_one(const int8_t* __restrict__ Q8, int64_
     // the owner of k flips x_k (when relinking, k leaves the candidates)
     const int kc = k / CW, kr = k - kc * CW;
     if (T == 32 || (kr >> 9) == warp) {
-      const int qkk = reinterpret_cast<const int8_t*>(diag)[k];
+      const int qkk = RL ? 0 : reinterpret_cast<const int8_t*>(diag)[k];
       flip_tree<0, E, E, RL>(key, sel, xm, kc * 16 + (kr & 15),
                              (2 * qkk - best.x) * (1 << kKeyBits), (kr >> 4) == g);
     }
@@ -708,7 +717,6 @@ relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
   __shared__ int2 rec[2][T / 32];
   __shared__ uint64_t xs[UBQP_MAX_N / 64];
   __shared__ uint4 spec_slots[spec_slot_count<T, C, R>()];
-  __shared__ uint4 diag[T * C];
   __shared__ unsigned long long ticket;
   Group<T> grp{rec, 0};
   if (err[1] != 0) return;  // Q failed its symmetry check: no walk
@@ -728,7 +736,8 @@ relink_block_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                        trace + p * ldt, xs};
     int64_t f0 = f[p];
     ascend_one<T, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
-                              nullptr, err, spec_slots, diag, Y ? Y + p * ldy : nullptr, grp, &a);
+                              nullptr, err, spec_slots, nullptr, Y ? Y + p * ldy : nullptr, grp,
+                              &a);
   }
 }
 
@@ -743,7 +752,6 @@ relink_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
                    unsigned long long* __restrict__ next) {
   __shared__ uint64_t xs_all[4][16];
   __shared__ uint4 spec_slots[4 * spec_slot_count<32, C, R>()];
-  __shared__ uint4 diag[4 * 32 * C];
   Group<32> grp;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (err[1] != 0) return;  // Q failed its symmetry check: no walk
@@ -760,8 +768,7 @@ relink_warp_kernel(const int8_t* __restrict__ Q8, int64_t ldq, int n, int W,
     int64_t f0 = f[p];
     ascend_one<32, C, R, true>(Q8, ldq, ldy, n, W, const_cast<uint64_t*>(X + p * W), &f0, 0,
                                nullptr, err,
-                               spec_slots + warp * spec_slot_count<32, C, R>(),
-                               diag + warp * (32 * C),
+                               spec_slots + warp * spec_slot_count<32, C, R>(), nullptr,
                                Y ? Y + p * ldy : nullptr, grp, &a);
   }
 }
