@@ -804,9 +804,10 @@ def main():
     inst.sync()
 
     # ---- roofline of the dominant kernel (ascent).  Per move the ascent reads
-    # one int8 row of Q (n bytes, L2-resident) and does 3n integer operations
-    # (each element's gain update, key and comparison), so its moves/s are
-    # bounded by min(L2 read rate / n, integer rate / 3n); both rates are
+    # one int8 row of Q (n bytes, L2-resident) and does 2n integer operations
+    # (each element's key update, half a comparison and, every other move, its
+    # selector's sign), so its moves/s are bounded by
+    # min(L2 read rate / n, integer rate / 2n); both rates are
     # measured here on this GPU (ubqp_peak_*).  The passers of the timed steps
     # are recounted untimed for the report.
     passers = 0
@@ -824,10 +825,10 @@ def main():
         pass
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    alu_peak = mp["ascent_update_tops"] * 1e12            # ops/s, 3 per element update
+    alu_peak = mp["ascent_update_tops"] * 1e12            # ops/s, 2 per element update
     l2_peak = mp["l2_read_gbs"] * 1e9                      # bytes/s
-    moves_roof = min(l2_peak / n, alu_peak / (3 * n))
-    l2_bound = l2_peak / n < alu_peak / (3 * n)
+    moves_roof = min(l2_peak / n, alu_peak / (2 * n))
+    l2_bound = l2_peak / n < alu_peak / (2 * n)
 
     def ascent_roofline(moves, secs):
         r = {"kernel": "ascent", "bound": "l2" if l2_bound else "alu",
@@ -837,15 +838,15 @@ def main():
             r.update(achieved=n * moves / secs / 1e9 if secs > 0 else None,
                      peak=l2_peak / 1e9, unit="GB/s (L2 read)")
         else:
-            r.update(achieved=3 * n * moves / secs / 1e12 if secs > 0 else None,
+            r.update(achieved=2 * n * moves / secs / 1e12 if secs > 0 else None,
                      peak=alu_peak / 1e12, unit="Tops/s (int32)")
         r["frac"] = r["achieved"] / r["peak"] if r["achieved"] else None
         r["peak_source"] = ("measured in this run on this GPU: the ascent's element update "
-                            "(dp4a + multiply-add + three-way max, 3 ops per element) at full "
-                            "occupancy" if not l2_bound else
+                            "(dp4a + half a three-way max + half a selector XOR, 2 ops per "
+                            "element) at full occupancy" if not l2_bound else
                             "measured in this run on this GPU: 16-byte L2 reads of a "
                             f"{mp['l2_buffer_bytes'] >> 20} MiB resident buffer")
-        r["work"] = f"{'n bytes' if l2_bound else '3n int32 ops'} per move, n = {n}"
+        r["work"] = f"{'n bytes' if l2_bound else '2n int32 ops'} per move, n = {n}"
         return r
 
     roof_asc = ascent_roofline(flips_timed, asc_s)

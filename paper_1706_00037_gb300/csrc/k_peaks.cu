@@ -1,7 +1,7 @@
 // k_peaks.cu -- measurement kernels for the rooflines of the ascent: the rate
 // at which the SMs read an L2-resident buffer, and the rate of the integer
 // instructions the ascent's per-element work is made of.  The steepest ascent
-// of the Pseudocode section reads one row of Q per move from L2 and does a few
+// of the Pseudocode section reads one row of Q per move from L2 and does two
 // integer operations per element; its roofline is the smaller of the L2 read
 // rate divided by the row bytes and the integer rate divided by the work per
 // move.  These kernels measure both rates on the device the library runs on;
@@ -41,9 +41,12 @@ l2_read_kernel(const uint4* __restrict__ buf, int64_t words, int reps, uint32_t*
 
 // kind 0: eight independent int32 multiply-add chains per thread (the plain
 // int32 instruction rate).  kind 1: the ascent's element update on sixteen
-// elements per thread -- per element y += d q (dp4a with d in the byte lane),
-// key = C + S y (multiply-add), and a running maximum folding two keys per
-// three-way max.
+// elements per thread -- per element one dp4a into its key, half a three-way
+// maximum (two keys folded at a time, two running maxima), and every other
+// iteration one XOR of its selector, as the climb turns them when a move's sign
+// differs from the last one's, about every other move.  Two instructions per
+// element.  The row word is new in every iteration and the selectors are kept in
+// registers, so nothing of it can be left out.
 template <int KIND>
 __global__ void __launch_bounds__(kPeakThreads, 4)
 int_rate_kernel(int64_t iters, uint32_t seed, uint32_t* sink) {
@@ -61,33 +64,33 @@ int_rate_kernel(int64_t iters, uint32_t seed, uint32_t* sink) {
     for (int i = 0; i < 8; ++i) out ^= (uint32_t)a[i];
   } else {
     constexpr int E = 16;
-    int y[E], S[E], Ck[E];
+    int key[E];
+    uint32_t sel[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      y[e] = (int)(seed + threadIdx.x + e);
-      S[e] = (e & 1) ? -128 : 128;
-      Ck[e] = 64 * (e - 8) + e;
+      key[e] = (int)(seed + threadIdx.x + e);
+      sel[e] = ((e + threadIdx.x) & 1 ? 0xC0u : 0x40u) << (8 * (e & 3));
     }
     int w = (int)(seed * 2654435761u + threadIdx.x);
-    int km = 0;
+    int best = 0;
     for (int64_t t = 0; t < iters; ++t) {
-      const int sel[4] = {(int)(t & 1) ? 0xFF : 0x01, (int)(t & 1) ? 0xFF00 : 0x0100,
-                          (int)(t & 1) ? 0xFF0000 : 0x010000,
-                          (int)(t & 1) ? (int)0xFF000000 : 0x01000000};
-      int k[4] = {INT_MIN, INT_MIN, INT_MIN, INT_MIN};
+      if (t & 1) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) sel[e] ^= 0x80u << (8 * (e & 3));
+      }
+      int k[2] = {INT_MIN, INT_MIN};
 #pragma unroll
       for (int e = 0; e < E; e += 2) {
-        y[e] = __dp4a(w, sel[e & 3], y[e]);
-        y[e + 1] = __dp4a(w, sel[(e + 1) & 3], y[e + 1]);
-        k[(e >> 1) & 3] = __vimax3_s32(k[(e >> 1) & 3], Ck[e] + S[e] * y[e],
-                                       Ck[e + 1] + S[e + 1] * y[e + 1]);
+        key[e] = __dp4a(w, (int)sel[e], key[e]);
+        key[e + 1] = __dp4a(w, (int)sel[e + 1], key[e + 1]);
+        k[(e >> 1) & 1] = __vimax3_s32(k[(e >> 1) & 1], key[e], key[e + 1]);
       }
-      km ^= max(max(k[0], k[1]), max(k[2], k[3]));
+      best ^= max(k[0], k[1]);
       w = w * 1664525 + 1013904223;
     }
-    out = (uint32_t)km;
+    out = (uint32_t)best;
 #pragma unroll
-    for (int e = 0; e < E; ++e) out ^= (uint32_t)y[e];
+    for (int e = 0; e < E; ++e) out ^= (uint32_t)key[e];
   }
   if (out == 0x9E3779B9u) sink[0] = out;
 }
@@ -124,7 +127,7 @@ int64_t ubqp_peak_int32_ops(int32_t kind, int64_t iters) {
   const int sms = ubqp::peak_grid();
   if (sms < 1 || (kind != 0 && kind != 1) || iters < 1) return 0;
   const int64_t threads = (int64_t)sms * 4 * ubqp::kPeakThreads;
-  return threads * iters * (kind == 0 ? 8 : 16 * 3);
+  return threads * iters * (kind == 0 ? 8 : 16 * 2);
 }
 
 int ubqp_peak_int32(int32_t kind, int64_t iters, uint32_t* sink_dev, void* stream) {
