@@ -891,6 +891,13 @@ cudaError_t launch_ascent_shaped(const ubqp_q* h, uint64_t* X, int64_t* f, const
   };
   const int64_t full = 10ll * h->sm_count;
 #define UBQP_C(TT, CC, RR, OCC) Climb<TT, CC, RR, OCC, TR>{}
+  // n <= 128: one launch, the climbs being as short as a launch that returns at once
+  // (33, 23 of 1600 starts, a few moves each: 24.2 us with both, 23.0; 100, 28 of
+  // 1600 30.3, 28.3; two launches are faster again from n = 200 on, 1380 of 8000
+  // starts 65.2 with one, 59.0 with two)
+  if (n <= 128)
+    return S > full ? UBQP_C(32, 1, 0, 10).launch(a, 0, INT64_MAX)
+                    : UBQP_C(32, 1, 0, 8).launch(a, 0, INT64_MAX);
   if (n <= 512) return two(UBQP_C(32, 1, 0, 8), UBQP_C(32, 1, 0, 10), full);
   if (n <= 1024) return two(UBQP_C(64, 1, 0, 8), UBQP_C(32, 2, 0, 8), full);
   if (n <= 1536) return tiers(UBQP_C(96, 1, 0, 7), UBQP_C(64, 2, 0, 8), UBQP_C(32, 3, 0, 6), full);
