@@ -142,24 +142,38 @@ __device__ __forceinline__ void emit_tile(const int8_t (*tile)[PT + 4], int rb, 
 // checks on them inside Q (aligned words and a funnel shift where rows are not).
 // What is left is the latency of a load phase and a store phase per block, five
 // blocks to an SM (eight, with 32 registers, measured slower).
-// The blocks walk the triangle of pairs along its diagonals, 2 x 2 tiles (a
-// super-tile pair (a, b), b = a + d mod sn for d = 0 .. sn / 2) at a time: blockIdx.y
-// = d sn + a, the last diagonal, d = sn / 2, only half as long.  Along a row, as
-// they ran before, a block's second tile lay 64 rows below the previous block's, so
-// that hundreds of blocks at once touched addresses a multiple of 64 n apart: at n =
-// 16384 and just below (strides of a power of two) 494 and 565 us against 444 and
-// 446 for the unpacked kernel before, 370 now; n = 12288 197 -> 180, n = 6001 and
-// 7000 the same.  The number of tiles is a multiple of four, so sn is even.
-template <bool W4>
+// Which pair a block takes.  Small squares: along the rows, the triangle folded
+// into a rectangle (tiles + 1, tiles / 2).  From DIAG_N on: along the diagonals, 2 x 2
+// tiles at a time (super-tiles (a, b), b = a + d mod sn for d = 0 .. sn / 2;
+// blockIdx.y = d sn + a, the last diagonal, d = sn / 2, only half as long).  Along a
+// row a block's second tile lies 64 rows below the previous block's, so hundreds of
+// blocks at once touch addresses a multiple of 64 rows apart, which costs the more
+// the longer the rows, most of all where they are a power of two.  Preparing, us, by
+// rows / by diagonals: n = 12288 197 / 179, n = 14336 309 / 255, n = 16383 566 / 375, n =
+// 16384 485 / 373 (446 and 444 before the packed forms).  The lines meet near n = 8000;
+// below, an evaluation right behind the preparation finds more of Q' in the L2 after
+// the rows (with 100 starts, n = 7000 136 / 139, n = 8192 161 / 159, n = 10240 223 /
+// 217).  The number of tiles is a multiple of four, so sn is even.
+// (Two kernels: with the choice made inside, 47 registers instead of 40, n = 16384
+// prepared in 525.)
+constexpr int DIAG_N = 8192;
+template <bool W4, bool DIAG>
 __global__ void __launch_bounds__(PTHREADS)
 prepare_pairs(const int8_t* __restrict__ Q, int n, int64_t ldq_in, int8_t* __restrict__ Q8,
               int64_t ldq, uint16_t* __restrict__ Qt, uint16_t* __restrict__ Qu, int n_tc,
               int32_t* __restrict__ rowsum, unsigned* __restrict__ flags) {
   pdl_enter();
   const int tiles = n_tc / PT;
-  const int sn = tiles / 2, a = (int)blockIdx.y % sn, b = (a + (int)blockIdx.y / sn) % sn;
-  const int bi = 2 * min(a, b) + (int)blockIdx.x / 2, bj = 2 * max(a, b) + (int)blockIdx.x % 2;
-  if (bi > bj) return;
+  int bi = blockIdx.y, bj = (int)blockIdx.x - 1;
+  if (DIAG) {
+    const int sn = tiles / 2, a = (int)blockIdx.y % sn, b = (a + (int)blockIdx.y / sn) % sn;
+    bi = 2 * min(a, b) + (int)blockIdx.x / 2;
+    bj = 2 * max(a, b) + (int)blockIdx.x % 2;
+    if (bi > bj) return;
+  } else if (bj < bi) {
+    bi = tiles - 1 - bi;
+    bj = tiles - 1 - (int)blockIdx.x;
+  }
   __shared__ __align__(16) int8_t tile[2][PT][PT + 4];  // T, then U
   const int t = threadIdx.x;
   const int nt = bi == bj ? 1 : 2;
@@ -260,25 +274,31 @@ first_derivative_bits(const int32_t* __restrict__ rowsum, int n, int W,
     reinterpret_cast<uint32_t*>(x0)[j >> 5] = bits;
 }
 
+template <bool W4, bool DIAG>
+cudaError_t launch_pairs(const int8_t* Q, int n, int64_t ldq_in, ubqp_q* h, cudaStream_t st) {
+  const int tiles = h->n_tc / PT, sn = tiles / 2;
+  const dim3 grid = DIAG ? dim3(4, sn * (sn + 1) / 2) : dim3(tiles + 1, sn);
+  return launch_pdl(prepare_pairs<W4, DIAG>, grid, dim3(PTHREADS), 0, st, Q, n, ldq_in, h->Q8,
+                    h->ldq, h->Qt, h->Qu, h->n_tc, h->rowsum, h->scratch_flags);
+}
+
 }  // namespace
 
 cudaError_t launch_prepare(const int8_t* Q, int n, int64_t ldq_in, ubqp_q* h,
                            cudaStream_t st) {
-  const int tiles = h->n_tc / PT;
   const int64_t work = std::max<int64_t>(h->n, (int64_t)h->n * (h->ldq - h->n_tc) / 16);
   prepare_clear<<<(unsigned)std::min<int64_t>((work + PTHREADS - 1) / PTHREADS,
                                               8ll * h->sm_count),
                   PTHREADS, 0, st>>>(h->rowsum, h->err, h->Q8, h->ldq, n, h->n_tc);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const int sn = tiles / 2;
-  const dim3 grid(4, sn * (sn + 1) / 2);
-  if (((uintptr_t)Q & 3) == 0 && (ldq_in & 3) == 0)
-    e = launch_pdl(prepare_pairs<true>, grid, dim3(PTHREADS), 0, st, Q, n, ldq_in, h->Q8, h->ldq,
-                   h->Qt, h->Qu, h->n_tc, h->rowsum, h->scratch_flags);
+  const bool w4 = ((uintptr_t)Q & 3) == 0 && (ldq_in & 3) == 0;
+  if (h->n_tc >= DIAG_N)
+    e = w4 ? launch_pairs<true, true>(Q, n, ldq_in, h, st)
+           : launch_pairs<false, true>(Q, n, ldq_in, h, st);
   else
-    e = launch_pdl(prepare_pairs<false>, grid, dim3(PTHREADS), 0, st, Q, n, ldq_in, h->Q8, h->ldq,
-                   h->Qt, h->Qu, h->n_tc, h->rowsum, h->scratch_flags);
+    e = w4 ? launch_pairs<true, false>(Q, n, ldq_in, h, st)
+           : launch_pairs<false, false>(Q, n, ldq_in, h, st);
   if (e != cudaSuccess) return e;
   return launch_pdl(first_derivative_bits, dim3((unsigned)((h->W * 64 + PTHREADS - 1) / PTHREADS)),
                     dim3(PTHREADS), 0, st, h->rowsum, n, h->W, h->x0);

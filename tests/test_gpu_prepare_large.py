@@ -12,7 +12,7 @@ from paper_1706_00037_gb300 import ubqp
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [1281, 4097, 16129, 16383, 16384])
+@pytest.mark.parametrize("n", [1281, 4097, 7936, 7937, 16129, 16383, 16384])
 def test_prepare_large(n):
     g = torch.Generator("cuda").manual_seed(n)
     Q = torch.randint(-100, 101, (n, n), dtype=torch.int8, device="cuda", generator=g)
