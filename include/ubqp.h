@@ -195,7 +195,9 @@ int ubqp_diversify_range(const ubqp_q* q, const uint64_t* x0_dev, int32_t mode,
  *        needs no workspace.
  *   path UBQP_EVAL_AUTO: UBQP_EVAL_TC_STAGED, except UBQP_EVAL_TC for
  *        n_pad <= 1024 (n rounded up to 256) with S >= 4096 (the faster of
- *        the two, measured).
+ *        the two, measured).  For n <= 128 with n S <= 2^18 and S <= 8192 it
+ *        launches one kernel with Q in shared memory in their place: the same
+ *        values, and the same workspace is asked for, which it leaves unused.
  * Returns UBQP_ERR_RANGE if the exactness bound fails (see top of file).
  */
 size_t ubqp_eval_workspace_size(const ubqp_q* q, int64_t S, int32_t path);
@@ -288,9 +290,9 @@ int ubqp_screen_apply(const int64_t* f_dev, int64_t S, const int64_t* gstats_dev
  *   listed starts run as one tensor-core product (bf16 Q, fp32 accumulation,
  *   exact), and the groups take the listed starts one at a time from a
  *   counter there as they finish (so long and short climbs even out over the
- *   SMs); with ws NULL or smaller the start-up sums the rows of Q on the CUDA
- *   cores and the starts are dealt round robin.  Results are identical either
- *   way.
+ *   SMs); with ws NULL or smaller, and for n <= 128 with S at most ten per SM,
+ *   the start-up sums the rows of Q on the CUDA cores and the starts are dealt
+ *   round robin.  Results are identical either way.
  */
 size_t ubqp_ascent_workspace_size(const ubqp_q* q, int64_t S);
 int ubqp_ascent(const ubqp_q* q, uint64_t* X_dev, int64_t* f_dev,
@@ -406,12 +408,13 @@ int ubqp_solve_rounds(const ubqp_q* q, const ubqp_params* p, int32_t R, uint64_t
  *   group shapes (threads x chunks that hold the largest n, one start per
  *   group, or packed: a launch per size class of the instances, each with the
  *   group shape for its n, on the internal streams, the instances above
- *   n = 4096 in launches of their own beside them), the evaluation paths, one merged launch for the start generation and the
- *   tensor-core evaluation of all instances (one persistent launch over the
- *   work units of every instance, largest first) or one launch per instance,
- *   the evaluation's schedule (at most 16, 12 or 8 K steps of 64 per work
- *   chunk) and the fork/join stream counts on this batch and keeps the
- *   fastest; drops a captured graph.  Synchronises `stream`.
+ *   n = 4096 in launches of their own beside them), the evaluation paths, one
+ *   merged launch for the start generation and the tensor-core evaluation of
+ *   all instances (one persistent launch over the work units of every
+ *   instance, largest first) or one launch per instance, the evaluation's
+ *   schedule (at most 16, 12 or 8 K steps of 64 per work chunk) and the fork/join
+ *   stream counts on this batch and keeps the fastest; drops a captured graph.
+ *   Synchronises `stream`.
  * ubqp_batch_capture -- records one run into a CUDA graph (after one plain
  *   run); later ubqp_batch_run calls replay it.  Synchronises `stream`.
  * ubqp_batch_result -- device pointers to instance i's best solution (W words)

@@ -477,7 +477,7 @@ size_t ubqp_ascent_workspace_size(const ubqp_q* q, int64_t S) {
 }
 
 // ubqp_ascent and ubqp_ascent_trace: the tensor-core start-up when the
-// workspace allows, then one ascent launch (traced when trace_dev is given).
+// workspace allows, then the ascent's launches (traced when trace_dev is given).
 static int ascent_impl(const ubqp_q* q, uint64_t* X_dev, int64_t* f_dev, const int32_t* idx_dev,
                        const int64_t* count_dev, int64_t S, int32_t max_flips,
                        int32_t* flips_dev, uint16_t* trace_dev, int64_t ldt, void* ws,

@@ -79,7 +79,7 @@ struct ubqp_batch {
   std::vector<int> alt_nchunks[2];
   // configuration (autotuned)
   int asc_T = 256, asc_C = 1, eval_path = UBQP_EVAL_TC, nstreams = 8;
-  bool packed = false;                   // packed ascent (sub-groups by n)
+  bool packed = false;                   // packed ascent (a launch per size class)
   int eval_kch = 16;                     // K steps per evaluation work chunk
   // the merged evaluation: start generation and the tensor-core evaluation of
   // every instance in one launch each (work lists for 16, 12 and 8 K steps)

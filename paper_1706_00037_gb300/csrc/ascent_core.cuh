@@ -12,9 +12,13 @@ namespace ubqp {
 namespace {
 
 constexpr int64_t kTimeoutNs = 20ll * 1000 * 1000 * 1000;  // per start
-// Runner-up rows copied one move ahead.  Measured at n = 7000 / 2500 / 1500
-// (passing starts of 1000 random ones): one row is 3-13% faster than none;
-// two or more cost more in reductions and copies than their hits save.
+// Runner-up rows that relinking copies one move ahead.  One against none, us, with
+// the present flip and reduction: one pair n = 1000 149 / 169, n = 4500 397 / 484,
+// n = 7500 640 / 793; 100 pairs 125 / 121, 342 / 334, 541 / 516; 256 pairs 128 / 127,
+// 432 / 383, 759 / 630.  So the copies pay while few blocks run, and a rule by the
+// number of pairs would gain above about one pair per SM.  (Climbs above n = 8192,
+// one against none: n = 9000, 11 starts 3245 / 2972, 544 starts 5382 / 4640; n =
+// 16384, 21 starts 6355 / 6895, 547 starts 10438 / 10255.)
 constexpr int kSpecRows = 1;
 // Starts per block of the one-warp kernels.
 constexpr int kWarps = 2;
@@ -846,8 +850,9 @@ struct Climb {
 // 40% of moves that hit saved (with and without: n = 1025, 510 starts 131 -> 113; 2500,
 // 542 starts 351 -> 270; 7000, 54 starts 1630 -> 1580, 641 starts 2567 -> 2192).
 //   all  few warps per start, and elements beyond n in as few threads as the
-//        registers allow (one warp up to n = 2560, 80 elements a thread), for lists that keep every SM busy: there the issue
-//        slots bound the climb, and the copies cost more than their hits save.
+//        registers allow (one warp up to n = 2560, 80 elements a thread), for lists
+//        that keep every SM busy: there the issue slots bound the climb, and the
+//        copies cost more than their hits save.
 //        (n = 2500, 3213 starts: two warps of 48 elements a thread 1059, one of 80
 //        996; n = 5000, 4469 starts: 96 threads of 64 5255, with 1144 elements
 //        beyond n, 160 of 32 4659; n = 1400: seven blocks per SM 662, six 634.)

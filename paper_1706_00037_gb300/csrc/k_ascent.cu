@@ -37,11 +37,11 @@
 // 7000, 54 starts: 737 cycles per move, 1.58 ms; 863 and 1.85 with y, S and C
 // registers).  The loads of the row are issued before anything else of the
 // move, its end test included; the selectors' flip and the owner's branches run
-// in their shadow.  Relinking, and climbs above n = 8192, take the fetch off the
-// chain where the move was predicted: every move also copies the row of the
-// reduction's runner-up into shared memory, and the next move is that row about
-// 40% of the time at n = 7000.  The other climbs make no such copies: they cost
-// more per move than the hits save.
+// in their shadow.  Relinking, climbs above n = 8192 and the unpacked batch climb's
+// short lists take the fetch off the chain where the move was predicted: every
+// move also copies the row of the reduction's runner-up into shared memory, and
+// the next move is that row about 40% of the time at n = 7000.  The other climbs
+// make no such copies: they cost more per move than the hits save.
 // With many starts the issue slots and the latency of 12 to 20 warps bound it
 // (n = 1400, 6069 starts: about 185 warp instructions per move, 91 cycles per
 // move and SM, 0.63 ms; 199 cycles and 1.38 ms with y, S and C registers).
@@ -64,8 +64,9 @@ cudaError_t launch_relink(const ubqp_q* h, const uint64_t* X, const int64_t* f, 
     if (e != cudaSuccess) return e;
   }
   // P is known here: up to one pair per SM the registers are sized for one
-  // block per SM (the shortest chain), above it for two (n = 5000, 256 pairs:
-  // see the launch rule of the ascent)
+  // block per SM (the shortest chain), above it for two, so that 256 pairs are one
+  // wave and not two (n = 4500, 256 pairs 674 us with y, S and C registers and one
+  // block per SM, 432 now; 150 pairs 394 and 342)
   const bool wide = P > h->sm_count;
 #define UBQP_RL(TT, CC, OCC) \
   return launch_relink_block<TT, CC, OCC>(h, X, f, G, P, Xb, fb, dist, trace, ldt, Y, next, st)
